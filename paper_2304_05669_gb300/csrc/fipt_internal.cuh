@@ -29,10 +29,13 @@ struct SceneConst {
 // Internal BVH node (64 bytes): both child boxes plus child references.
 // A reference >= 0 is an internal node; < 0 is the leaf ~ref (one triangle
 // at that sorted position).
-//   a = (c0.lo.x, c0.hi.x, c0.lo.y, c0.hi.y)
-//   b = (c1.lo.x, c1.hi.x, c1.lo.y, c1.hi.y)
+//   a = (c0.lo.x, c0.lo.y, c0.hi.x, c0.hi.y)
+//   b = (c1.lo.x, c1.lo.y, c1.hi.x, c1.hi.y)
 //   c = (c0.lo.z, c0.hi.z, c1.lo.z, c1.hi.z)
 //   d = (child0, child1, -, -)
+// x and y stand side by side so that the slab test's differences and
+// products are two-wide float operations on register pairs as loaded
+// (node_test).
 struct __align__(16) BvhNode {
     float4 a, b, c;
     int4 d;
@@ -288,8 +291,8 @@ __device__ __forceinline__ float u24f(uint32_t w) {
 // kz = dominant axis of d, kx/ky the others (swapped when d[kz] < 0 to keep
 // the winding), shear S.
 struct TraceRay {
-    float ox, oy, oz;
-    float ix, iy, iz;       // 1/d for the slab tests
+    float2 mxy, mz;         // minus the origin: (-ox, -oy), (-oz, -oz)
+    float2 ixy, iz;         // 1/d for the slab tests: (1/dx, 1/dy), (1/dz, 1/dz)
     float Sx, Sy, Sz;
     int k;                  // kx | ky << 2 | kz << 4
 };
@@ -301,11 +304,13 @@ __device__ __forceinline__ float pick3(float x, float y, float z, int k) {
 __device__ __forceinline__ TraceRay make_ray(float ox, float oy, float oz, float dx, float dy,
                                              float dz) {
     TraceRay r;
-    r.ox = ox; r.oy = oy; r.oz = oz;
+    r.mxy = make_float2(-ox, -oy);
+    r.mz = make_float2(-oz, -oz);
     const float tiny = 1e-20f;
-    r.ix = 1.0f / (fabsf(dx) < tiny ? copysignf(tiny, dx) : dx);
-    r.iy = 1.0f / (fabsf(dy) < tiny ? copysignf(tiny, dy) : dy);
-    r.iz = 1.0f / (fabsf(dz) < tiny ? copysignf(tiny, dz) : dz);
+    r.ixy = make_float2(1.0f / (fabsf(dx) < tiny ? copysignf(tiny, dx) : dx),
+                        1.0f / (fabsf(dy) < tiny ? copysignf(tiny, dy) : dy));
+    const float iz = 1.0f / (fabsf(dz) < tiny ? copysignf(tiny, dz) : dz);
+    r.iz = make_float2(iz, iz);
     const float ax = fabsf(dx), ay = fabsf(dy), az = fabsf(dz);
     int kz = (ax >= ay && ax >= az) ? 0 : (ay >= az ? 1 : 2);
     int kx = kz == 2 ? 0 : kz + 1;
@@ -314,7 +319,9 @@ __device__ __forceinline__ TraceRay make_ray(float ox, float oy, float oz, float
     if (dkz < 0.0f) { int t = kx; kx = ky; ky = t; }
     r.Sx = pick3(dx, dy, dz, kx) / dkz;
     r.Sy = pick3(dx, dy, dz, ky) / dkz;
-    r.Sz = 1.0f / dkz;
+    // 1/d of the dominant axis again, but for a direction with no component
+    // the slab test's reciprocal takes as it is
+    r.Sz = fabsf(dkz) < tiny ? 1.0f / dkz : pick3(r.ixy.x, r.ixy.y, iz, kz);
     r.k = kx | (ky << 2) | (kz << 4);
     return r;
 }
@@ -326,9 +333,9 @@ __device__ __forceinline__ TraceRay make_ray(float ox, float oy, float oz, float
 __device__ __forceinline__ bool tri_intersect(const TraceRay& r, float4 p0, float4 p1, float4 p2,
                                               float& t, bool& front) {
     const int kx = r.k & 3, ky = (r.k >> 2) & 3, kz = (r.k >> 4) & 3;
-    const float Ax0 = p0.x - r.ox, Ay0 = p0.y - r.oy, Az0 = p0.z - r.oz;
-    const float Bx0 = p1.x - r.ox, By0 = p1.y - r.oy, Bz0 = p1.z - r.oz;
-    const float Cx0 = p2.x - r.ox, Cy0 = p2.y - r.oy, Cz0 = p2.z - r.oz;
+    const float Ax0 = p0.x + r.mxy.x, Ay0 = p0.y + r.mxy.y, Az0 = p0.z + r.mz.x;
+    const float Bx0 = p1.x + r.mxy.x, By0 = p1.y + r.mxy.y, Bz0 = p1.z + r.mz.x;
+    const float Cx0 = p2.x + r.mxy.x, Cy0 = p2.y + r.mxy.y, Cz0 = p2.z + r.mz.x;
     const float Akz = pick3(Ax0, Ay0, Az0, kz), Bkz = pick3(Bx0, By0, Bz0, kz),
                 Ckz = pick3(Cx0, Cy0, Cz0, kz);
     const float Ax = fmaf(-r.Sx, Akz, pick3(Ax0, Ay0, Az0, kx));
@@ -362,31 +369,36 @@ __device__ __forceinline__ bool tri_intersect(const TraceRay& r, float4 p0, floa
 // just below tmax: then another triangle's hit within that gap is kept.
 __device__ __forceinline__ void node_test(const TraceRay& r, const BvhNode& n, float tmax,
                                           bool& hit0, bool& hit1, float& t0, float& t1) {
-    const float ox = r.ox, oy = r.oy, oz = r.oz;
-    const float a0 = (n.a.x - ox) * r.ix, a1 = (n.a.y - ox) * r.ix;
-    const float a2 = (n.a.z - oy) * r.iy, a3 = (n.a.w - oy) * r.iy;
-    const float a4 = (n.c.x - oz) * r.iz, a5 = (n.c.y - oz) * r.iz;
-    const float b0 = (n.b.x - ox) * r.ix, b1 = (n.b.y - ox) * r.ix;
-    const float b2 = (n.b.z - oy) * r.iy, b3 = (n.b.w - oy) * r.iy;
-    const float b4 = (n.c.z - oz) * r.iz, b5 = (n.c.w - oz) * r.iz;
+    const float2 al = __fmul2_rn(__fadd2_rn(make_float2(n.a.x, n.a.y), r.mxy), r.ixy);
+    const float2 ah = __fmul2_rn(__fadd2_rn(make_float2(n.a.z, n.a.w), r.mxy), r.ixy);
+    const float2 az = __fmul2_rn(__fadd2_rn(make_float2(n.c.x, n.c.y), r.mz), r.iz);
+    const float2 bl = __fmul2_rn(__fadd2_rn(make_float2(n.b.x, n.b.y), r.mxy), r.ixy);
+    const float2 bh = __fmul2_rn(__fadd2_rn(make_float2(n.b.z, n.b.w), r.mxy), r.ixy);
+    const float2 bz = __fmul2_rn(__fadd2_rn(make_float2(n.c.z, n.c.w), r.mz), r.iz);
     const float robust = 1.0000005f;
-    const float n0 = fmaxf(fmaxf(fminf(a0, a1), fminf(a2, a3)), fmaxf(fminf(a4, a5), 0.0f));
-    const float f0 = fminf(fminf(fmaxf(a0, a1), fmaxf(a2, a3)), fminf(fmaxf(a4, a5), tmax));
-    const float n1 = fmaxf(fmaxf(fminf(b0, b1), fminf(b2, b3)), fmaxf(fminf(b4, b5), 0.0f));
-    const float f1 = fminf(fminf(fmaxf(b0, b1), fmaxf(b2, b3)), fminf(fmaxf(b4, b5), tmax));
+    const float n0 = fmaxf(fmaxf(fminf(al.x, ah.x), fminf(al.y, ah.y)), fmaxf(fminf(az.x, az.y), 0.0f));
+    const float f0 = fminf(fminf(fmaxf(al.x, ah.x), fmaxf(al.y, ah.y)), fminf(fmaxf(az.x, az.y), tmax));
+    const float n1 = fmaxf(fmaxf(fminf(bl.x, bh.x), fminf(bl.y, bh.y)), fmaxf(fminf(bz.x, bz.y), 0.0f));
+    const float f1 = fminf(fminf(fmaxf(bl.x, bh.x), fmaxf(bl.y, bh.y)), fminf(fmaxf(bz.x, bz.y), tmax));
     hit0 = n0 <= f0 * robust;
     hit1 = n1 <= f1 * robust;
     t0 = n0;
     t1 = n1;
 }
 
+// A node's record in two 32-byte loads (sm_100's widest), one per sector:
+// half the load instructions and fewer L1 wavefronts (79 -> 72 % of the data
+// pipe's peak on the room) than four 16-byte loads.  Records are 64-byte
+// aligned: the node arrays start 256-byte aligned in the scene's workspace.
 __device__ __forceinline__ BvhNode load_node(const BvhNode* nodes, int i) {
-    const float4* p = reinterpret_cast<const float4*>(nodes + i);
+    const BvhNode* p = nodes + i;
     BvhNode n;
-    n.a = __ldg(p + 0);
-    n.b = __ldg(p + 1);
-    n.c = __ldg(p + 2);
-    n.d = __ldg(reinterpret_cast<const int4*>(p + 3));
+    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(n.a.x), "=f"(n.a.y), "=f"(n.a.z), "=f"(n.a.w), "=f"(n.b.x), "=f"(n.b.y), "=f"(n.b.z), "=f"(n.b.w)
+        : "l"(p));
+    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8+32];"
+        : "=f"(n.c.x), "=f"(n.c.y), "=f"(n.c.z), "=f"(n.c.w), "=r"(n.d.x), "=r"(n.d.y), "=r"(n.d.z), "=r"(n.d.w)
+        : "l"(p));
     return n;
 }
 
@@ -451,88 +463,48 @@ __device__ __forceinline__ float3 voxel_lookup(const SceneView& sc, float px, fl
 }
 
 // ---------------------------------------------------------------- traversal
-// Traversal stack entries per thread.  k_trace and k_camera keep the stack
-// in shared memory (a [depth][thread] column per block); the bake (k_bake,
-// k_serve_bake) and the refinement's traversal keep it in a per-thread
-// local-memory array.  A ray whose stack would overflow drops the far
-// child it could not push (that subtree is not searched) and sets
+// Traversal stack entries per thread, in a per-thread local-memory array: a
+// kernel that walks reserves no shared memory, and the SM's unified L1 /
+// shared storage serves as cache for the nodes and for the stack entries in
+// use.  Entry 0 is the end mark, so a pop needs no emptiness test, and the
+// array has room for the pushes between two checks of its fill (WALK_UNROLL).
+// A ray found with more than STACK_DEPTH entries at a check loses the ones
+// above it (those subtrees are not searched) and sets
 // FIPT_DEV_STACK_OVERFLOW in the device status word.
 #ifndef FIPT_STACK_DEPTH
 #define FIPT_STACK_DEPTH 32
 #endif
 constexpr int STACK_DEPTH = FIPT_STACK_DEPTH;
+#ifndef FIPT_WALK_UNROLL
+#define FIPT_WALK_UNROLL 8       // node visits between two checks of the walk's bounds
+#endif
+constexpr int WALK_UNROLL = FIPT_WALK_UNROLL;
+constexpr int STACK_SLOTS = 1 + STACK_DEPTH + WALK_UNROLL;
 constexpr float FINF = __builtin_huge_valf();
 
+// Closest hit so far: its distance and its leaf, ~leaf when the ray met the
+// back face, FIPT_DONE when there is none.
 struct BestHit {
     float t;
-    int leaf;
-    int orig;
-    bool front;
+    int code;
+    __device__ __forceinline__ bool any() const { return code != FIPT_DONE; }
+    __device__ __forceinline__ bool front() const { return code >= 0; }
+    __device__ __forceinline__ int leaf() const { return code >= 0 ? code : ~code; }   // of a hit
 };
 
-// Closest hit of one ray; `stack` is this thread's column of the shared
-// stack (element k at stack[k * STRIDE]).  A full stack raises the
-// overflow bit (the ray loses that subtree).
-template <int STRIDE>
-__device__ __forceinline__ void closest_hit(const SceneView& sc, const TraceRay& r, int skip,
-                                            int* stack, BestHit& best, int32_t* status) {
-    best.t = FINF;
-    best.leaf = -1;
-    best.orig = 0x7fffffff;
-    best.front = false;
-    if (sc.T == 0) return;
-    int node = 0, sp = 0, steps = 0;
-    while (node != FIPT_DONE) {
-        while (node >= 0) {
-            if (node >= sc.n_inner || ++steps > sc.max_steps) {
-                atomicOr(status, node >= sc.n_inner ? FIPT_DEV_BAD_NODE : FIPT_DEV_STEP_LIMIT);
-                return;
-            }
-            const BvhNode n = load_node(sc.nodes, node);
-            bool h0, h1;
-            float t0, t1;
-            node_test(r, n, best.t, h0, h1, t0, t1);
-            if (h0 && h1) {
-                const bool first0 = t0 <= t1;
-                if (sp < STACK_DEPTH) {
-                    stack[sp * STRIDE] = first0 ? n.d.y : n.d.x;
-                    ++sp;
-                } else {
-                    atomicOr(status, FIPT_DEV_STACK_OVERFLOW);
-                }
-                node = first0 ? n.d.x : n.d.y;
-            } else if (h0) {
-                node = n.d.x;
-            } else if (h1) {
-                node = n.d.y;
-            } else {
-                node = sp > 0 ? stack[--sp * STRIDE] : FIPT_DONE;
-            }
-        }
-        while (node < 0 && node != FIPT_DONE) {
-            const int leaf = ~node;
-            if (leaf >= sc.T || ++steps > sc.max_steps) {
-                atomicOr(status, leaf >= sc.T ? FIPT_DEV_BAD_NODE : FIPT_DEV_STEP_LIMIT);
-                return;
-            }
-            const float4 p0 = __ldg(sc.tris + 3 * leaf);
-            const int orig = __float_as_int(p0.w);
-            if (orig != skip) {
-                const float4 p1 = __ldg(sc.tris + 3 * leaf + 1), p2 = __ldg(sc.tris + 3 * leaf + 2);
-                float t;
-                bool fr;
-                if (tri_intersect(r, p0, p1, p2, t, fr) &&
-                    (t < best.t || (t == best.t && orig < best.orig))) {
-                    best.t = t;
-                    best.leaf = leaf;
-                    best.orig = orig;
-                    best.front = fr;
-                }
-            }
-            node = sp > 0 ? stack[--sp * STRIDE] : FIPT_DONE;
-        }
+// A lane's walk: the node or leaf reference it is at (FIPT_DONE: none left),
+// a parked leaf (-1: none), its stack pointer, and the node and leaf visits
+// it has made.
+struct Walk {
+    int node, parked, sp, steps;
+    __device__ __forceinline__ bool idle() const { return node == FIPT_DONE && parked < 0; }
+    __device__ __forceinline__ void start(const SceneView& sc) {
+        node = sc.T > 0 ? 0 : FIPT_DONE;
+        parked = -1;
+        sp = 1;
+        steps = 0;
     }
-}
+};
 
 // Counters of an instrumented walk: node visits, triangle tests, deepest
 // stack.
@@ -542,63 +514,84 @@ struct WalkStats {
 };
 
 // One round of a warp's speculative walk (Aila and Laine 2009).  Every lane
-// descends inner nodes; a lane that reaches a leaf parks it (pleaf) and,
-// with SPECULATE, keeps descending until every lane holds a leaf or is
-// done; the parked leaves, and leaves that follow them on the stack, are
-// then tested.  A lane whose walk is over has node == FIPT_DONE and
-// pleaf < 0; lanes without a ray call with that state and just vote.  All
-// 32 lanes of the warp must call it together.  `stack` is the lane's
-// column of the shared stack (entry k at stack[k * STRIDE]).  A lane with
-// stop_on_hit ends its walk at the first triangle that improves `best`.
-template <int STRIDE, bool STATS, bool SPECULATE>
-__device__ __forceinline__ void warp_walk(const SceneView& sc, const TraceRay& r, int skip, BestHit& best,
-                                          int& node, int& pleaf, int& sp, int& steps, int* stack,
-                                          int32_t* status, WalkStats& ws, bool stop_on_hit = false) {
+// descends inner nodes; a lane that reaches a leaf parks it and keeps
+// descending until every lane holds a leaf or is done; the parked leaves,
+// and leaves that follow them on the stack, are then tested.  Lanes without
+// a ray call idle and just vote.  All 32 lanes of the warp call it together.
+// stack[0] is FIPT_DONE.  A lane with stop_on_hit ends its walk at the first
+// triangle that improves `best`.
+//
+// The walk is bound by the instructions it issues and, next, by L1
+// wavefronts (78 % of the data pipe's peak).  So its guards (node references
+// in range, stack room, the step limit of a valid tree) are acted on once
+// per WALK_UNROLL visits: a reference out of range is never followed
+// meanwhile (it fails the one unsigned compare that tells nodes from
+// leaves), and the stack has room for WALK_UNROLL more pushes.  With the
+// two-wide slab test and the 32-byte node loads, whose effects depend on one
+// another through the 32 registers the bake has, the room's bake (2^18
+// points x 64 samples) went from 33.1 to 28.8 ms and the floor's (2^19 x 64)
+// from 57.5 to 50.0 ms, 17 % fewer instructions, all results bit-identical.
+// Unrolling by 2 / 4 / 8 / 12 / 16 / 24: 30.7 / 29.7 / 28.7 / 28.6 / 28.5 /
+// 32.5 ms (24 outgrows the instruction cache); without the 32-byte loads 29.3
+// at 8, without the two-wide test 30.4.  Measured slower: the guards and the
+// pops as selects instead of branches (29.2), a sample queue per lane so that
+// lanes wait less for the warp's slowest ray (2 to 8 samples: 33-35 ms; the
+// lanes drift apart and no longer visit the same nodes).
+template <bool STATS>
+__device__ __forceinline__ void warp_walk(const SceneView& sc, const TraceRay& r, int skip, BestHit& best, Walk& w,
+                                          int* stack, int32_t* status, WalkStats& ws, bool stop_on_hit = false) {
     for (;;) {
-        if (node >= 0 && (SPECULATE || pleaf < 0)) {
-            if (node >= sc.n_inner || ++steps > sc.max_steps) {
-                atomicOr(status, node >= sc.n_inner ? FIPT_DEV_BAD_NODE : FIPT_DEV_STEP_LIMIT);
-                node = FIPT_DONE;
-                pleaf = -1;
-                sp = 0;
-            } else {
-                const BvhNode n = load_node(sc.nodes, node);
+        bool more = true;
+#pragma unroll
+        for (int u = 0; u < WALK_UNROLL; ++u) {
+            if ((unsigned)w.node < (unsigned)sc.n_inner) {
+                const BvhNode n = load_node(sc.nodes, w.node);
                 if (STATS) ++ws.nodes;
+                ++w.steps;
                 bool h0, h1;
                 float t0, t1;
                 node_test(r, n, best.t, h0, h1, t0, t1);
                 if (h0 && h1) {
                     const bool first0 = t0 <= t1;
-                    if (sp < STACK_DEPTH) {
-                        stack[sp * STRIDE] = first0 ? n.d.y : n.d.x;
-                        ++sp;
-                        if (STATS) ws.max_sp = max(ws.max_sp, sp);
-                    } else {
-                        atomicOr(status, FIPT_DEV_STACK_OVERFLOW);
-                    }
-                    node = first0 ? n.d.x : n.d.y;
+                    stack[w.sp] = first0 ? n.d.y : n.d.x;
+                    ++w.sp;
+                    if (STATS) ws.max_sp = max(ws.max_sp, w.sp - 1);
+                    w.node = first0 ? n.d.x : n.d.y;
                 } else if (h0) {
-                    node = n.d.x;
+                    w.node = n.d.x;
                 } else if (h1) {
-                    node = n.d.y;
+                    w.node = n.d.y;
                 } else {
-                    node = sp > 0 ? stack[--sp * STRIDE] : FIPT_DONE;
+                    w.node = stack[--w.sp];
                 }
             }
+            if ((unsigned)w.node > 0x80000000u && w.parked < 0) {    // park the first leaf found
+                w.parked = ~w.node;
+                w.node = stack[--w.sp];
+            }
+            more = __any_sync(0xffffffffu, w.parked < 0 && (unsigned)w.node < (unsigned)sc.n_inner);
+            if (!more) break;                                         // every lane has a leaf or is done
         }
-        if (node < 0 && node != FIPT_DONE && pleaf < 0) {   // park the first leaf found
-            pleaf = ~node;
-            node = sp > 0 ? stack[--sp * STRIDE] : FIPT_DONE;
+        if (w.node >= sc.n_inner || w.steps > sc.max_steps || w.sp > STACK_DEPTH + 1) {
+            if (w.node >= sc.n_inner || w.steps > sc.max_steps) {
+                atomicOr(status, w.node >= sc.n_inner ? FIPT_DEV_BAD_NODE : FIPT_DEV_STEP_LIMIT);
+                w.node = FIPT_DONE;
+                w.parked = -1;
+                w.sp = 0;
+                w.steps = 0;
+            } else {
+                atomicOr(status, FIPT_DEV_STACK_OVERFLOW);
+                w.sp = STACK_DEPTH + 1;
+            }
         }
-        if (!__any_sync(0xffffffffu, pleaf < 0 && node >= 0)) break;   // every lane has a leaf or is done
+        if (!more) break;
     }
-    while (pleaf >= 0) {
-        const int leaf = pleaf;
-        pleaf = -1;
-        if (leaf >= sc.T || ++steps > sc.max_steps) {
-            atomicOr(status, leaf >= sc.T ? FIPT_DEV_BAD_NODE : FIPT_DEV_STEP_LIMIT);
-            node = FIPT_DONE;
-            sp = 0;
+    while (w.parked >= 0) {
+        const int leaf = w.parked;
+        w.parked = -1;
+        if (leaf >= (int)sc.T || ++w.steps > sc.max_steps) {
+            atomicOr(status, leaf >= (int)sc.T ? FIPT_DEV_BAD_NODE : FIPT_DEV_STEP_LIMIT);
+            w.node = FIPT_DONE;
             break;
         }
         const float4 p0 = __ldg(sc.tris + 3 * leaf);
@@ -608,22 +601,38 @@ __device__ __forceinline__ void warp_walk(const SceneView& sc, const TraceRay& r
             const float4 p1 = __ldg(sc.tris + 3 * leaf + 1), p2 = __ldg(sc.tris + 3 * leaf + 2);
             float t;
             bool fr;
-            if (tri_intersect(r, p0, p1, p2, t, fr) && (t < best.t || (t == best.t && orig < best.orig))) {
-                best.t = t;
-                best.leaf = leaf;
-                best.orig = orig;
-                best.front = fr;
-                if (stop_on_hit) {
-                    node = FIPT_DONE;
-                    sp = 0;
-                    break;
+            if (tri_intersect(r, p0, p1, p2, t, fr)) {
+                bool better = t < best.t;
+                if (t == best.t)                  // a tie goes to the lower triangle index
+                    better = !best.any() || orig < __float_as_int(__ldg(&sc.tris[3 * best.leaf()].w));
+                if (better) {
+                    best.t = t;
+                    best.code = fr ? leaf : ~leaf;
+                    if (stop_on_hit) {
+                        w.node = FIPT_DONE;
+                        break;
+                    }
                 }
             }
         }
-        if (node < 0 && node != FIPT_DONE) {      // the next entry is a leaf too
-            pleaf = ~node;
-            node = sp > 0 ? stack[--sp * STRIDE] : FIPT_DONE;
+        if ((unsigned)w.node > 0x80000000u) {     // the next entry is a leaf too
+            w.parked = ~w.node;
+            w.node = stack[--w.sp];
         }
     }
 }
 
+// Closest hit of one ray per lane; lanes without a ray pass has_ray = false.
+// All 32 lanes of the warp call it together.
+__device__ __forceinline__ void closest_hit(const SceneView& sc, const TraceRay& r, bool has_ray, int skip,
+                                            BestHit& best, int32_t* status) {
+    int stack[STACK_SLOTS];
+    stack[0] = FIPT_DONE;
+    WalkStats ws;
+    Walk w;
+    w.start(sc);
+    if (!has_ray) w.node = FIPT_DONE;
+    best.t = FINF;
+    best.code = FIPT_DONE;
+    while (__any_sync(0xffffffffu, !w.idle())) warp_walk<false>(sc, r, skip, best, w, stack, status, ws);
+}

@@ -454,8 +454,8 @@ __device__ __forceinline__ Box leaf_box(const float4* tris, int leaf) {
 __device__ __forceinline__ Box node_box(const BvhNode* nodes, int i) {
     const float4* p = reinterpret_cast<const float4*>(nodes + i);
     const float4 a = __ldcg(p), b = __ldcg(p + 1), c = __ldcg(p + 2);
-    return Box{fminf(a.x, b.x), fminf(a.z, b.z), fminf(c.x, c.z),
-               fmaxf(a.y, b.y), fmaxf(a.w, b.w), fmaxf(c.y, c.w)};
+    return Box{fminf(a.x, b.x), fminf(a.y, b.y), fminf(c.x, c.z),
+               fmaxf(a.z, b.z), fmaxf(a.w, b.w), fmaxf(c.y, c.w)};
 }
 
 __global__ void k_refit(BvhNode* nodes, const float4* __restrict__ tris,
@@ -476,8 +476,8 @@ __global__ void k_refit(BvhNode* nodes, const float4* __restrict__ tris,
         const Box b0 = ch.x < 0 ? leaf_box(tris, ~ch.x) : node_box(nodes, ch.x);
         const Box b1 = ch.y < 0 ? leaf_box(tris, ~ch.y) : node_box(nodes, ch.y);
         float4* q = reinterpret_cast<float4*>(nodes + p);
-        __stcg(q + 0, make_float4(b0.lx, b0.hx, b0.ly, b0.hy));
-        __stcg(q + 1, make_float4(b1.lx, b1.hx, b1.ly, b1.hy));
+        __stcg(q + 0, make_float4(b0.lx, b0.ly, b0.hx, b0.hy));
+        __stcg(q + 1, make_float4(b1.lx, b1.ly, b1.hx, b1.hy));
         __stcg(q + 2, make_float4(b0.lz, b0.hz, b1.lz, b1.hz));
         p = parent[p];
     }
@@ -520,8 +520,8 @@ __device__ __forceinline__ void child_boxes(const BvhNode* nodes, int n, Box& b0
     const float4* q = reinterpret_cast<const float4*>(nodes + n);
     const float4 a = __ldcg(q), b = __ldcg(q + 1), c = __ldcg(q + 2);
     ch = __ldcg(reinterpret_cast<const int4*>(q + 3));
-    b0 = Box{a.x, a.z, c.x, a.y, a.w, c.y};
-    b1 = Box{b.x, b.z, c.z, b.y, b.w, c.w};
+    b0 = Box{a.x, a.y, c.x, a.z, a.w, c.y};
+    b1 = Box{b.x, b.y, c.z, b.z, b.w, c.w};
 }
 
 // Per-warp tables of the dynamic programme (shared memory).
@@ -629,11 +629,11 @@ __device__ void restructure_warp(BvhNode* nodes, int32_t* parent, int32_t* leaf_
             if (par >= 0) {
                 BvhNode& R = rec[par];
                 if (side == 0) {
-                    R.a = make_float4(b.lx, b.hx, b.ly, b.hy);
+                    R.a = make_float4(b.lx, b.ly, b.hx, b.hy);
                     R.c.x = b.lz; R.c.y = b.hz;
                     R.d.x = r;
                 } else {
-                    R.b = make_float4(b.lx, b.hx, b.ly, b.hy);
+                    R.b = make_float4(b.lx, b.ly, b.hx, b.hy);
                     R.c.z = b.lz; R.c.w = b.hz;
                     R.d.y = r;
                 }
@@ -782,8 +782,8 @@ __global__ void k_relabel_leaves(int32_t* leaf_parent, const int32_t* __restrict
 __global__ void k_single(BvhNode* nodes, const float4* __restrict__ tris, int32_t* range) {
     const Box b = leaf_box(tris, 0);
     const float inf = __int_as_float(0x7f800000);
-    nodes[0].a = make_float4(b.lx, b.hx, b.ly, b.hy);
-    nodes[0].b = make_float4(inf, -inf, inf, -inf);
+    nodes[0].a = make_float4(b.lx, b.ly, b.hx, b.hy);
+    nodes[0].b = make_float4(inf, inf, -inf, -inf);
     nodes[0].c = make_float4(b.lz, b.hz, inf, -inf);
     nodes[0].d = make_int4(~0, ~0, 0, 0);
     range[0] = 0; range[1] = 0; range[2] = 0;
@@ -800,9 +800,9 @@ __global__ void k_export_boxes(const BvhNode* __restrict__ nodes, int64_t n, flo
     }
     if (!out) return;
     out[6 * i + 0] = fminf(nd.a.x, nd.b.x);
-    out[6 * i + 1] = fminf(nd.a.z, nd.b.z);
+    out[6 * i + 1] = fminf(nd.a.y, nd.b.y);
     out[6 * i + 2] = fminf(nd.c.x, nd.c.z);
-    out[6 * i + 3] = fmaxf(nd.a.y, nd.b.y);
+    out[6 * i + 3] = fmaxf(nd.a.z, nd.b.z);
     out[6 * i + 4] = fmaxf(nd.a.w, nd.b.w);
     out[6 * i + 5] = fmaxf(nd.c.y, nd.c.w);
 }

@@ -428,7 +428,8 @@ template <bool STATS>
 __global__ void __launch_bounds__(RF_TRACE_THREADS, FIPT_RF_TRACE_MINB)
 k_rf_trace(SceneView sc, RfState st, int w, int32_t* status, unsigned long long* stats) {
     constexpr unsigned FULL = 0xffffffffu;
-    int stack[STACK_DEPTH];             // local memory, as the stage-1 bake's
+    int stack[STACK_SLOTS];             // local memory, as the stage-1 bake's
+    stack[0] = FIPT_DONE;
     const uint32_t* __restrict__ queue = st.tq[w & 1];
     uint32_t* cnt = st.cnt + 4 * w;
     const uint32_t n = cnt[0];
@@ -439,16 +440,18 @@ k_rf_trace(SceneView sc, RfState st, int w, int32_t* status, unsigned long long*
     TraceRay r = make_ray(0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 1.0f);
     BestHit best;
     best.t = FINF;
-    best.leaf = -1;
-    best.orig = 0x7fffffff;
-    best.front = false;
-    int node = FIPT_DONE, pleaf = -1, sp = 0, steps = 0;
+    best.code = FIPT_DONE;
+    Walk wk;
+    wk.start(sc);
+    wk.node = FIPT_DONE;
     WalkStats ws;
     unsigned long long n_rays = 0;
     for (;;) {
-        const bool idle = node == FIPT_DONE && pleaf < 0;
+        const bool idle = wk.idle();
         if (idle && rid >= 0) {
-            st.hit[rid] = make_int4(__float_as_int(best.t), best.leaf, best.orig, best.front ? 1 : 0);
+            st.hit[rid] = best.any() ? make_int4(__float_as_int(best.t), best.leaf(),
+                                                 __float_as_int(__ldg(&sc.tris[3 * best.leaf()].w)), best.front() ? 1 : 0)
+                                     : make_int4(__float_as_int(best.t), -1, 0x7fffffff, 0);
             rid = -1;
         }
         const bool need = idle && !drained;
@@ -468,12 +471,8 @@ k_rf_trace(SceneView sc, RfState st, int w, int32_t* status, unsigned long long*
                     r = make_ray(o.x, o.y, o.z, d.x, d.y, d.z);
                     skip = __float_as_int(o.w);
                     best.t = d.w;
-                    best.leaf = -1;
-                    best.orig = 0x7fffffff;
-                    best.front = false;
-                    sp = 0;
-                    steps = 0;
-                    node = sc.T > 0 ? 0 : FIPT_DONE;
+                    best.code = FIPT_DONE;
+                    wk.start(sc);
                     if (STATS) ++n_rays;
                     shadow = (rid & 1) != 0;
                     if (shadow) {                  // settle the target first
@@ -485,13 +484,11 @@ k_rf_trace(SceneView sc, RfState st, int w, int32_t* status, unsigned long long*
                         if (STATS) ++ws.tris;
                         if (orig != skip &&
                             tri_intersect(r, p0, __ldg(sc.tris + 3 * tgt + 1), __ldg(sc.tris + 3 * tgt + 2), t, fr) &&
-                            (t < best.t || (t == best.t && orig < best.orig))) {
+                            t <= best.t) {         // no hit yet: a tie with t_max is one
                             best.t = t;
-                            best.leaf = tgt;
-                            best.orig = orig;
-                            best.front = fr;
+                            best.code = fr ? tgt : ~tgt;
                         } else {
-                            node = FIPT_DONE;      // unlit whatever else the ray meets
+                            wk.node = FIPT_DONE;      // unlit whatever else the ray meets
                         }
                     }
                 } else {
@@ -499,8 +496,7 @@ k_rf_trace(SceneView sc, RfState st, int w, int32_t* status, unsigned long long*
                 }
             }
         }
-        warp_walk<1, STATS, true>(sc, r, skip, best, node, pleaf, sp, steps, stack, status, ws,
-                                                 shadow);
+        warp_walk<STATS>(sc, r, skip, best, wk, stack, status, ws, shadow);
     }
     if (STATS) {
         atomicAdd(&stats[0], n_rays);

@@ -1,13 +1,9 @@
 // Ray traversal kernels: closest hit, pinhole first hits, query compaction
 // and the bake of the factorized shading terms (Eq. 6-7, Eq. 9, Sec. 6).
 //
-// Traversal is a per-thread stack walk of the binary LBVH in "while-while"
-// form (inner nodes until a leaf, then leaves until an inner node).  The
-// first-hit kernels keep the stack in shared memory, laid out
-// [depth][thread] so that the threads of a warp touch consecutive banks;
-// the bake keeps it in local memory (see bake_item).  Node (64 B) and
-// triangle (48 B) reads are 16-byte vector loads through the read-only
-// path.
+// Traversal is warp_walk (fipt_internal.cuh): a stack walk of the binary
+// tree, a ray per lane, the warp's lanes in step between inner nodes and
+// leaves, the stack in local memory.
 #include "fipt_internal.cuh"
 #include "render_math.cuh"
 
@@ -19,24 +15,24 @@ __global__ void __launch_bounds__(TRACE_THREADS)
 k_trace(SceneView sc, const float* __restrict__ orig, const float* __restrict__ dir, int64_t n,
         const int32_t* __restrict__ skip, int32_t* __restrict__ hit_tri, float* __restrict__ hit_t,
         int32_t* __restrict__ hit_front, int32_t* status) {
-    __shared__ int stk[STACK_DEPTH * TRACE_THREADS];
     const int64_t i = blockIdx.x * (int64_t)TRACE_THREADS + threadIdx.x;
-    if (i >= n) return;
-    const TraceRay r = make_ray(orig[3 * i], orig[3 * i + 1], orig[3 * i + 2], dir[3 * i],
-                                dir[3 * i + 1], dir[3 * i + 2]);
+    const bool on = i < n;
+    TraceRay r = make_ray(0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 1.0f);
+    if (on) r = make_ray(orig[3 * i], orig[3 * i + 1], orig[3 * i + 2], dir[3 * i], dir[3 * i + 1], dir[3 * i + 2]);
     BestHit b;
-    closest_hit<TRACE_THREADS>(sc, r, skip ? skip[i] : -1, stk + threadIdx.x, b, status);
-    hit_tri[i] = b.leaf >= 0 ? b.orig : -1;
+    closest_hit(sc, r, on, on && skip ? skip[i] : -1, b, status);
+    if (!on) return;
+    hit_tri[i] = b.any() ? __float_as_int(__ldg(&sc.tris[3 * b.leaf()].w)) : -1;
     hit_t[i] = b.t;
-    hit_front[i] = b.leaf >= 0 && b.front ? 1 : 0;
+    hit_front[i] = b.any() && b.front() ? 1 : 0;
 }
 
 __global__ void __launch_bounds__(TRACE_THREADS)
 k_camera(SceneView sc, const float* __restrict__ cams, int W, int H, int64_t P,
          fipt_query* __restrict__ out, int32_t* __restrict__ valid, int32_t* status) {
-    __shared__ int stk[STACK_DEPTH * TRACE_THREADS];
-    const int64_t p = blockIdx.x * (int64_t)TRACE_THREADS + threadIdx.x;
-    if (p >= P) return;
+    const int64_t slot = blockIdx.x * (int64_t)TRACE_THREADS + threadIdx.x;
+    const bool on = slot < P;
+    const int64_t p = on ? slot : P - 1;
     const int64_t wh = (int64_t)W * H;
     const int v = (int)(p / wh);
     const int64_t rem = p - v * wh;
@@ -58,15 +54,17 @@ k_camera(SceneView sc, const float* __restrict__ cams, int W, int H, int64_t P,
     dx *= dl; dy *= dl; dz *= dl;
     const TraceRay r = make_ray(c[0], c[1], c[2], dx, dy, dz);
     BestHit b;
-    closest_hit<TRACE_THREADS>(sc, r, -1, stk + threadIdx.x, b, status);
+    closest_hit(sc, r, on, -1, b, status);
+    if (!on) return;
     fipt_query qr;
-    if (b.leaf < 0) {
+    if (!b.any()) {
         for (int a = 0; a < 3; ++a) { qr.x[a] = 0.0f; qr.n[a] = 0.0f; qr.wo[a] = 0.0f; }
         qr.tri = -1;
         valid[p] = 0;
     } else {
-        const float4 p0 = __ldg(sc.tris + 3 * b.leaf), p1 = __ldg(sc.tris + 3 * b.leaf + 1),
-                     p2 = __ldg(sc.tris + 3 * b.leaf + 2);
+        const int leaf = b.leaf();
+        const float4 p0 = __ldg(sc.tris + 3 * leaf), p1 = __ldg(sc.tris + 3 * leaf + 1),
+                     p2 = __ldg(sc.tris + 3 * leaf + 2);
         const float e1x = p1.x - p0.x, e1y = p1.y - p0.y, e1z = p1.z - p0.z;
         const float e2x = p2.x - p0.x, e2y = p2.y - p0.y, e2z = p2.z - p0.z;
         float nx = e1y * e2z - e1z * e2y, ny = e1z * e2x - e1x * e2z, nz = e1x * e2y - e1y * e2x;
@@ -75,7 +73,7 @@ k_camera(SceneView sc, const float* __restrict__ cams, int W, int H, int64_t P,
         qr.x[0] = c[0] + b.t * dx; qr.x[1] = c[1] + b.t * dy; qr.x[2] = c[2] + b.t * dz;
         qr.n[0] = sg * nx; qr.n[1] = sg * ny; qr.n[2] = sg * nz;
         qr.wo[0] = -dx; qr.wo[1] = -dy; qr.wo[2] = -dz;
-        qr.tri = b.orig;
+        qr.tri = __float_as_int(p0.w);
         valid[p] = 1;
     }
     out[p] = qr;
@@ -176,9 +174,6 @@ constexpr int BAKE_THREADS = FIPT_BAKE_THREADS;
 #ifndef FIPT_BAKE_REFILL
 #define FIPT_BAKE_REFILL 32      // lanes that must be waiting before a warp draws new rays (32: all that still sample)
 #endif
-#ifndef FIPT_BAKE_SPECULATE
-#define FIPT_BAKE_SPECULATE 1    // keep walking inner nodes while other lanes look for a leaf
-#endif
 
 // Bakes one (point, lobe) pair per lane: lobe 0 is the diffuse term, lobe
 // k+1 roughness level k.  Each lane walks its pair's samples in order and
@@ -196,11 +191,7 @@ constexpr int BAKE_THREADS = FIPT_BAKE_THREADS;
 //    alike (8 % faster on the building floor than refilling at 28);
 //  * speculation (Aila and Laine 2009): a lane that reaches a leaf parks
 //    it and keeps descending inner nodes until every lane has a leaf;
-//  * leaves are then tested together.
-// The traversal stack is a per-thread array in local memory, not a shared
-// memory column: the bake then reserves no shared memory and the SM's
-// unified L1 / shared storage serves as cache for the nodes and for the
-// stack entries actually in use.
+//  * leaves are then tested together (warp_walk).
 // FLAGS: 1 = environment light for misses, 2 = voxel radiance cache (each
 // used only where the pair's scene has one, so a launch over chunks of
 // several scenes takes the union of their flags).
@@ -211,7 +202,8 @@ __device__ __forceinline__ void bake_item(const SceneView& sc, const fipt_query*
                                           float* __restrict__ Ls0, float* __restrict__ Ls1,
                                           int32_t* status, unsigned long long* stats) {
     constexpr unsigned FULL = 0xffffffffu;
-    int stack[STACK_DEPTH];
+    int stack[STACK_SLOTS];
+    stack[0] = FIPT_DONE;
     float nx = 0.0f, ny = 0.0f, nz = 1.0f, wox = 0.0f, woy = 0.0f, woz = 1.0f;
     float px = 0.0f, py = 0.0f, pz = 0.0f;
     int skip = -1;
@@ -252,37 +244,41 @@ __device__ __forceinline__ void bake_item(const SceneView& sc, const fipt_query*
     float acc0x = 0, acc0y = 0, acc0z = 0, acc1x = 0, acc1y = 0, acc1z = 0;
     float wF0 = 1.0f, wF1 = 0.0f;
     float rdx = 0.0f, rdy = 0.0f, rdz = 1.0f;     // current ray direction (environment lookups)
-    int s = 0, node = FIPT_DONE, pleaf = -1, sp = 0, steps = 0;
+    int s = 0;
     bool active = false;
     TraceRay r;
     BestHit best;
-    best.leaf = -1;
-    unsigned long long n_rays = 0, n_nodes = 0, n_tris = 0;
-    int max_sp = 0;
+    best.code = FIPT_DONE;
+    Walk w;
+    w.start(sc);
+    w.node = FIPT_DONE;
+    WalkStats ws;
+    unsigned long long n_rays = 0;
 
     for (;;) {
         // ---------------- refill: gather finished rays, draw new ones together
-        const bool idle = node == FIPT_DONE && pleaf < 0;
+        const bool idle = w.idle();
         const bool need = idle && (active || s < S);
         const unsigned m_need = __ballot_sync(FULL, need);
         const unsigned m_busy = __ballot_sync(FULL, !idle);
         if ((m_need | m_busy) == 0) break;
         if (m_need != 0 && (m_busy == 0 || __popc(m_need) >= FIPT_BAKE_REFILL) && need) {
             if (active) {
-                bool lit = best.leaf >= 0;
+                bool lit = best.any();
                 float lx = 0.0f, ly = 0.0f, lz = 0.0f;
                 if (lit) {
-                    const float4 le = __ldg(sc.shade + 2 * best.leaf);
+                    const int leaf = best.leaf();
+                    const float4 le = __ldg(sc.shade + 2 * leaf);
                     float3 ca;
                     if ((FLAGS & 2) && sc.vox) {
                         ca = voxel_lookup(sc, ox + best.t * rdx, oy + best.t * rdy, oz + best.t * rdz);
                     } else {
-                        const float4 c4 = __ldg(sc.shade + 2 * best.leaf + 1);
+                        const float4 c4 = __ldg(sc.shade + 2 * leaf + 1);
                         ca = make_float3(c4.x, c4.y, c4.z);
                     }
-                    lx = (best.front ? le.x : 0.0f) + ca.x;
-                    ly = (best.front ? le.y : 0.0f) + ca.y;
-                    lz = (best.front ? le.z : 0.0f) + ca.z;
+                    lx = (best.front() ? le.x : 0.0f) + ca.x;
+                    ly = (best.front() ? le.y : 0.0f) + ca.y;
+                    lz = (best.front() ? le.z : 0.0f) + ca.z;
                 } else if ((FLAGS & 1) && sc.env) {
                     const float3 e = env_lookup(sc, rdx, rdy, rdz);
                     lx = e.x; ly = e.y; lz = e.z;
@@ -339,89 +335,14 @@ __device__ __forceinline__ void bake_item(const SceneView& sc, const fipt_query*
                 r = make_ray(ox, oy, oz, dx, dy, dz);
                 if (FLAGS) { rdx = dx; rdy = dy; rdz = dz; }
                 best.t = FINF;
-                best.leaf = -1;
-                best.orig = 0x7fffffff;
-                best.front = false;
-                sp = 0;
-                steps = 0;
-                node = sc.T > 0 ? 0 : FIPT_DONE;
+                best.code = FIPT_DONE;
+                w.start(sc);
                 active = true;
                 if (STATS) ++n_rays;
                 break;
             }
         }
-        // ---------------- inner nodes (speculative)
-        // (the same walk as warp_walk in fipt_internal.cuh, written out here:
-        // calling warp_walk from this kernel changes its register allocation
-        // and measured 3.8 % slower, with bit-identical results)
-        for (;;) {
-            if (node >= 0 && (FIPT_BAKE_SPECULATE || pleaf < 0)) {
-                if (node >= sc.n_inner || ++steps > sc.max_steps) {
-                    atomicOr(status, node >= sc.n_inner ? FIPT_DEV_BAD_NODE : FIPT_DEV_STEP_LIMIT);
-                    node = FIPT_DONE;
-                    pleaf = -1;
-                    sp = 0;
-                } else {
-                    const BvhNode n = load_node(sc.nodes, node);
-                    if (STATS) ++n_nodes;
-                    bool h0, h1;
-                    float t0, t1;
-                    node_test(r, n, best.t, h0, h1, t0, t1);
-                    if (h0 && h1) {
-                        const bool first0 = t0 <= t1;
-                        if (sp < STACK_DEPTH) {
-                            stack[sp] = first0 ? n.d.y : n.d.x;
-                            ++sp;
-                            if (STATS) max_sp = max(max_sp, sp);
-                        } else {
-                            atomicOr(status, FIPT_DEV_STACK_OVERFLOW);
-                        }
-                        node = first0 ? n.d.x : n.d.y;
-                    } else if (h0) {
-                        node = n.d.x;
-                    } else if (h1) {
-                        node = n.d.y;
-                    } else {
-                        node = sp > 0 ? stack[--sp] : FIPT_DONE;
-                    }
-                }
-            }
-            if (node < 0 && node != FIPT_DONE && pleaf < 0) {   // park the first leaf found
-                pleaf = ~node;
-                node = sp > 0 ? stack[--sp] : FIPT_DONE;
-            }
-            if (!__any_sync(FULL, pleaf < 0 && node >= 0)) break;   // every lane has a leaf or is done
-        }
-        // ---------------- leaves
-        while (pleaf >= 0) {
-            const int leaf = pleaf;
-            pleaf = -1;
-            if (leaf >= sc.T || ++steps > sc.max_steps) {
-                atomicOr(status, leaf >= sc.T ? FIPT_DEV_BAD_NODE : FIPT_DEV_STEP_LIMIT);
-                node = FIPT_DONE;
-                sp = 0;
-                break;
-            }
-            const float4 p0 = __ldg(sc.tris + 3 * leaf);
-            const int orig = __float_as_int(p0.w);
-            if (orig != skip) {
-                if (STATS) ++n_tris;
-                const float4 p1 = __ldg(sc.tris + 3 * leaf + 1), p2 = __ldg(sc.tris + 3 * leaf + 2);
-                float t;
-                bool fr;
-                if (tri_intersect(r, p0, p1, p2, t, fr) &&
-                    (t < best.t || (t == best.t && orig < best.orig))) {
-                    best.t = t;
-                    best.leaf = leaf;
-                    best.orig = orig;
-                    best.front = fr;
-                }
-            }
-            if (node < 0 && node != FIPT_DONE) {      // the next entry is a leaf too
-                pleaf = ~node;
-                node = sp > 0 ? stack[--sp] : FIPT_DONE;
-            }
-        }
+        warp_walk<STATS>(sc, r, skip, best, w, stack, status, ws);
     }
 
     if (valid) {
@@ -439,9 +360,9 @@ __device__ __forceinline__ void bake_item(const SceneView& sc, const fipt_query*
     }
     if (STATS) {
         atomicAdd(&stats[0], n_rays);
-        atomicAdd(&stats[1], n_nodes);
-        atomicAdd(&stats[2], n_tris);
-        atomicMax(&stats[3], (unsigned long long)max_sp);
+        atomicAdd(&stats[1], ws.nodes);
+        atomicAdd(&stats[2], ws.tris);
+        atomicMax(&stats[3], (unsigned long long)ws.max_sp);
     }
 }
 
