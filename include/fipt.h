@@ -448,8 +448,8 @@ fipt_status fipt_render_grad_scale(int64_t N, const double* grad_loss, float* g_
  * (-1 = none, ignored), pixel p's index at tri[p * tri_stride] (i32; 1 for
  * a plain array, 10 to read the tri field of fipt_query records); Lr, Lgt
  * [P,3] f32.  Outputs: err_sum [T] f64
- * = sum of ||Lr - Lgt||^2 over the triangle's pixels, summed in pixel
- * order; count [T] i32.  Pixels are grouped by a stable radix sort on the
+ * = sum of ||Lr - Lgt||^2 over the triangle's pixels, summed in FP64 in a
+ * fixed order; count [T] i32.  Pixels are grouped by a stable radix sort on the
  * triangle index held in the workspace. */
 fipt_status fipt_tri_error_workspace_size(int64_t P, int64_t T, size_t* bytes);
 fipt_status fipt_tri_error(const int32_t* tri, int64_t tri_stride, const float* Lr,
