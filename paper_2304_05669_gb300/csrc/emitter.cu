@@ -58,20 +58,26 @@ __global__ void k_debug_divide(DivN d, const uint32_t* __restrict__ i, int64_t c
 }
 
 // IDX: uint32_t when T * n < 2^32 (the sample index splits by the
-// multiply-high division above), int64_t otherwise.  A block stages its
-// PTS_THREADS points in shared memory and writes them as float4 (the
-// block's 12 * PTS_THREADS bytes start 16-byte aligned when x is).
+// multiply-high division above), int64_t otherwise.  Bound by the
+// instructions of a sample's ten Philox rounds and its square root, then by
+// the 12 bytes written, so a thread takes PTS_PER consecutive samples: the
+// index is divided and the triangle loaded once, and the block's points,
+// contiguous in x, leave shared memory in one bulk copy (x 16-byte aligned)
+// instead of by loads and stores.  204,546,400 points (100 on each triangle
+// of the floor): 1,062 -> 828 us (363 us at the copy rate), one point
+// per thread and float4 stores before.
 constexpr int PTS_THREADS = 256;
+constexpr int PTS_PER = 4;
+constexpr int PTS_BLOCK = PTS_THREADS * PTS_PER;
 
 template <class IDX>
 __global__ void __launch_bounds__(PTS_THREADS)
 k_emit_points(const float4* __restrict__ tris, const int32_t* __restrict__ inv, int64_t T, int n, DivN dn,
               uint2 key, uint32_t rid, float* __restrict__ x) {
-    __shared__ float4 buf[3 * PTS_THREADS / 4];
-    float* sb = reinterpret_cast<float*>(buf);
+    __shared__ __align__(128) float sb[3 * PTS_BLOCK];
     const int64_t total = T * n;
-    const int64_t base = (int64_t)blockIdx.x * PTS_THREADS;
-    const int64_t i = base + threadIdx.x;
+    const int64_t base = (int64_t)blockIdx.x * PTS_BLOCK;
+    const int64_t i = base + PTS_PER * threadIdx.x;
     if (i < total) {
         IDX t;
         if constexpr (sizeof(IDX) == 4) {
@@ -79,24 +85,48 @@ k_emit_points(const float4* __restrict__ tris, const int32_t* __restrict__ inv, 
         } else {
             t = (IDX)i / (IDX)n;
         }
-        const uint32_t j = (uint32_t)((IDX)i - t * (IDX)n);
-        const int leaf = inv[t];
-        const float4 p0 = __ldg(tris + 3 * leaf), p1 = __ldg(tris + 3 * leaf + 1), p2 = __ldg(tris + 3 * leaf + 2);
-        const uint4 w = philox4x32_10(make_uint4((uint32_t)t, j, EMIT_LANE, rid), key);
-        const float u1 = u24f(w.x), u2 = u24f(w.y);
-        const float r1 = sqrtf(u1);
-        const float b0 = 1.0f - r1, b1 = r1 * (1.0f - u2), b2 = r1 * u2;
-        sb[3 * threadIdx.x + 0] = b0 * p0.x + b1 * p1.x + b2 * p2.x;
-        sb[3 * threadIdx.x + 1] = b0 * p0.y + b1 * p1.y + b2 * p2.y;
-        sb[3 * threadIdx.x + 2] = b0 * p0.z + b1 * p1.z + b2 * p2.z;
+        int j = (int)((IDX)i - t * (IDX)n);
+        int leaf = inv[t];
+        float4 p0 = __ldg(tris + 3 * leaf), p1 = __ldg(tris + 3 * leaf + 1), p2 = __ldg(tris + 3 * leaf + 2);
+        float v[3 * PTS_PER];
+#pragma unroll
+        for (int q = 0; q < PTS_PER; ++q) {
+            if (q > 0 && ++j == n) {                       // the next triangle
+                j = 0;
+                if ((int64_t)++t < T) {
+                    leaf = inv[t];
+                    p0 = __ldg(tris + 3 * leaf);
+                    p1 = __ldg(tris + 3 * leaf + 1);
+                    p2 = __ldg(tris + 3 * leaf + 2);
+                }
+            }
+            const uint4 w = philox4x32_10(make_uint4((uint32_t)t, (uint32_t)j, EMIT_LANE, rid), key);
+            const float u1 = u24f(w.x), u2 = u24f(w.y);
+            const float r1 = sqrtf(u1);
+            const float b0 = 1.0f - r1, b1 = r1 * (1.0f - u2), b2 = r1 * u2;
+            v[3 * q + 0] = b0 * p0.x + b1 * p1.x + b2 * p2.x;
+            v[3 * q + 1] = b0 * p0.y + b1 * p1.y + b2 * p2.y;
+            v[3 * q + 2] = b0 * p0.z + b1 * p1.z + b2 * p2.z;
+        }
+        float4* dst = reinterpret_cast<float4*>(sb + 3 * PTS_PER * threadIdx.x);
+#pragma unroll
+        for (int q = 0; q < 3 * PTS_PER / 4; ++q) dst[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
     }
-    __syncthreads();
-    const int64_t here = total - base < PTS_THREADS ? total - base : PTS_THREADS;
-    if (here == PTS_THREADS && (reinterpret_cast<uintptr_t>(x) & 15) == 0) {
-        float4* dst = reinterpret_cast<float4*>(x + 3 * base);
-        if (threadIdx.x < 3 * PTS_THREADS / 4) dst[threadIdx.x] = buf[threadIdx.x];
+    const int64_t here = total - base < PTS_BLOCK ? total - base : PTS_BLOCK;
+    if (here == PTS_BLOCK && (reinterpret_cast<uintptr_t>(x) & 15) == 0) {     // the same for the whole block
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            const uint32_t src = (uint32_t)__cvta_generic_to_shared(sb);
+            asm volatile(
+                "cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n"
+                "cp.async.bulk.commit_group;\n"
+                "cp.async.bulk.wait_group.read 0;" ::"l"(x + 3 * base), "r"(src), "r"((uint32_t)sizeof(sb))
+                : "memory");
+        }
     } else {
-        for (int k = threadIdx.x; k < 3 * here; k += PTS_THREADS) x[3 * base + k] = sb[k];
+        __syncthreads();
+        for (int64_t k = threadIdx.x; k < 3 * here; k += PTS_THREADS) x[3 * base + k] = sb[k];
     }
 }
 
@@ -472,10 +502,10 @@ extern "C" fipt_status fipt_emitter_sample_points(fipt_scene* s, uint64_t seed, 
     const uint2 key = make_uint2((uint32_t)seed, (uint32_t)(seed >> 32));
     const DivN dn = div_by((uint32_t)n_per_tri);
     if (n < ((int64_t)1 << 32))
-        FIPT_LAUNCH(k_emit_points<uint32_t>, blocks(n, PTS_THREADS), PTS_THREADS, 0,
+        FIPT_LAUNCH(k_emit_points<uint32_t>, blocks(n, PTS_BLOCK), PTS_THREADS, 0,
                     static_cast<cudaStream_t>(stream), s->tris, s->inv, s->T, n_per_tri, dn, key, request_id, x);
     else
-        FIPT_LAUNCH(k_emit_points<int64_t>, blocks(n, PTS_THREADS), PTS_THREADS, 0,
+        FIPT_LAUNCH(k_emit_points<int64_t>, blocks(n, PTS_BLOCK), PTS_THREADS, 0,
                     static_cast<cudaStream_t>(stream), s->tris, s->inv, s->T, n_per_tri, dn, key, request_id, x);
     FIPT_LAUNCHED("emitter sample points");
     return FIPT_OK;
