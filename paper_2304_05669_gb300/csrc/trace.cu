@@ -4,6 +4,8 @@
 // Traversal is warp_walk (fipt_internal.cuh): a stack walk of the binary
 // tree, a ray per lane, the warp's lanes in step between inner nodes and
 // leaves, the stack in local memory.
+#include <algorithm>
+
 #include "fipt_internal.cuh"
 #include "render_math.cuh"
 
@@ -171,9 +173,6 @@ k_compact(const fipt_query* __restrict__ in, const int32_t* __restrict__ valid, 
 constexpr int BAKE_THREADS = FIPT_BAKE_THREADS;
 
 
-#ifndef FIPT_BAKE_REFILL
-#define FIPT_BAKE_REFILL 32      // lanes that must be waiting before a warp draws new rays (32: all that still sample)
-#endif
 
 // Bakes one (point, lobe) pair per lane: lobe 0 is the diffuse term, lobe
 // k+1 roughness level k.  Each lane walks its pair's samples in order and
@@ -181,26 +180,29 @@ constexpr int BAKE_THREADS = FIPT_BAKE_THREADS;
 // scheduling).  All 32 lanes of the warp stay in the loop until every lane
 // is done (lanes without a pair, `valid` false, just vote), because three
 // warp-level decisions keep the lanes doing the same work at the same time:
-//  * refill: a lane whose ray has finished waits until FIPT_BAKE_REFILL
-//    lanes (or all remaining lanes) are waiting; they then gather their
-//    results and draw their next rays together, so the Philox stream,
-//    direction sampling and ray set-up run with many lanes active.  With
-//    the default (every lane) the lanes draw the same sample index
-//    together, and as the samples are jittered strata of one grid their
-//    rays leave through the same cell of directions and walk the tree
-//    alike (8 % faster on the building floor than refilling at 28);
+//  * refill: a lane whose ray has finished waits until every lane's has;
+//    they then gather their results and draw their next rays together, so
+//    the Philox stream, direction sampling and ray set-up run with all lanes
+//    active, and the lanes draw the same sample index: as the samples are
+//    jittered strata of one grid their rays leave through the same cell of
+//    directions and walk the tree alike (8 % faster on the building floor
+//    than refilling at 28);
 //  * speculation (Aila and Laine 2009): a lane that reaches a leaf parks
 //    it and keeps descending inner nodes until every lane has a leaf;
 //  * leaves are then tested together (warp_walk).
 // FLAGS: 1 = environment light for misses, 2 = voxel radiance cache (each
 // used only where the pair's scene has one, so a launch over chunks of
 // several scenes takes the union of their flags).
-template <bool STATS, int FLAGS>
+// SPLIT: G consecutive lanes (a power of two) share a pair: lane g of them
+// draws samples g, g + G, ..., and after each round every one of them adds
+// the round's G contributions in sample order, with the same operations on
+// the same values as one lane would, so the results are the same bits.
+template <bool STATS, int FLAGS, bool SPLIT>
 __device__ __forceinline__ void bake_item(const SceneView& sc, const fipt_query* __restrict__ q,
                                           const int64_t p, const int lobe, const bool valid,
                                           const BakeArgs& A, float* __restrict__ Ld,
                                           float* __restrict__ Ls0, float* __restrict__ Ls1,
-                                          int32_t* status, unsigned long long* stats) {
+                                          int32_t* status, unsigned long long* stats, const int G = 1) {
     constexpr unsigned FULL = 0xffffffffu;
     int stack[STACK_SLOTS];
     stack[0] = FIPT_DONE;
@@ -244,7 +246,8 @@ __device__ __forceinline__ void bake_item(const SceneView& sc, const fipt_query*
     float acc0x = 0, acc0y = 0, acc0z = 0, acc1x = 0, acc1y = 0, acc1z = 0;
     float wF0 = 1.0f, wF1 = 0.0f;
     float rdx = 0.0f, rdy = 0.0f, rdz = 1.0f;     // current ray direction (environment lookups)
-    int s = 0;
+    const int in_group = SPLIT ? (int)(threadIdx.x & (G - 1)) : 0;
+    int s = in_group;
     bool active = false;
     TraceRay r;
     BestHit best;
@@ -257,15 +260,11 @@ __device__ __forceinline__ void bake_item(const SceneView& sc, const fipt_query*
 
     for (;;) {
         // ---------------- refill: gather finished rays, draw new ones together
-        const bool idle = w.idle();
-        const bool need = idle && (active || s < S);
-        const unsigned m_need = __ballot_sync(FULL, need);
-        const unsigned m_busy = __ballot_sync(FULL, !idle);
-        if ((m_need | m_busy) == 0) break;
-        if (m_need != 0 && (m_busy == 0 || __popc(m_need) >= FIPT_BAKE_REFILL) && need) {
+        if (!__any_sync(FULL, !w.idle())) {
+            float lx = 0.0f, ly = 0.0f, lz = 0.0f;
+            bool lit = false;
             if (active) {
-                bool lit = best.any();
-                float lx = 0.0f, ly = 0.0f, lz = 0.0f;
+                lit = best.any();
                 if (lit) {
                     const int leaf = best.leaf();
                     const float4 le = __ldg(sc.shade + 2 * leaf);
@@ -284,21 +283,36 @@ __device__ __forceinline__ void bake_item(const SceneView& sc, const fipt_query*
                     lx = e.x; ly = e.y; lz = e.z;
                     lit = true;
                 }
-                if (lit) {
-                    if (lobe == 0) {
-                        acc0x += lx; acc0y += ly; acc0z += lz;
-                    } else {
-                        acc0x += lx * wF0; acc0y += ly * wF0; acc0z += lz * wF0;
-                        acc1x += lx * wF1; acc1y += ly * wF1; acc1z += lz * wF1;
-                    }
-                }
                 active = false;
             }
+            if (SPLIT) {
+                const float w0 = lit ? wF0 : 0.0f, w1 = lit ? wF1 : 0.0f;     // an unlit sample adds zeros
+                for (int g = 0; g < G; ++g) {
+                    const int from = (int)(threadIdx.x & 31) - in_group + g;
+                    const float gx = __shfl_sync(FULL, lx, from), gy = __shfl_sync(FULL, ly, from),
+                                gz = __shfl_sync(FULL, lz, from);
+                    if (lobe == 0) {
+                        acc0x += gx; acc0y += gy; acc0z += gz;
+                    } else {
+                        const float g0 = __shfl_sync(FULL, w0, from), g1 = __shfl_sync(FULL, w1, from);
+                        acc0x = fmaf(gx, g0, acc0x); acc0y = fmaf(gy, g0, acc0y); acc0z = fmaf(gz, g0, acc0z);
+                        acc1x = fmaf(gx, g1, acc1x); acc1y = fmaf(gy, g1, acc1y); acc1z = fmaf(gz, g1, acc1z);
+                    }
+                }
+            } else if (lit) {
+                if (lobe == 0) {
+                    acc0x += lx; acc0y += ly; acc0z += lz;
+                } else {
+                    acc0x = fmaf(lx, wF0, acc0x); acc0y = fmaf(ly, wF0, acc0y); acc0z = fmaf(lz, wF0, acc0z);
+                    acc1x = fmaf(lx, wF1, acc1x); acc1y = fmaf(ly, wF1, acc1y); acc1z = fmaf(lz, wF1, acc1z);
+                }
+            }
+            if (!__any_sync(FULL, s < S)) break;
             while (s < S) {
                 const uint4 rnd = philox4x32_10(make_uint4(pid, (uint32_t)s, (uint32_t)lobe, A.request_id), A.key);
                 float u1 = u24f(rnd.x), u2 = u24f(rnd.y);
                 strat_uv((uint32_t)s, S, lobe == 0 ? A.nx_d : A.nx_s, u1, u2);
-                ++s;
+                s += SPLIT ? G : 1;
                 float sn, cs;
                 sincospif(2.0f * u2, &sn, &cs);
                 float dx, dy, dz;
@@ -345,7 +359,7 @@ __device__ __forceinline__ void bake_item(const SceneView& sc, const fipt_query*
         warp_walk<STATS>(sc, r, skip, best, w, stack, status, ws);
     }
 
-    if (valid) {
+    if (valid && (!SPLIT || in_group == 0)) {
         const float fs = (float)(S > 0 ? S : 1);
         if (lobe == 0) {
             Ld[3 * p + 0] = acc0x / fs;
@@ -366,20 +380,21 @@ __device__ __forceinline__ void bake_item(const SceneView& sc, const fipt_query*
     }
 }
 
-// A warp holds 32 consecutive points of one lobe; consecutive warps cycle
-// through the lobes of the same 32 points.
-template <bool STATS, int FLAGS>
+// A warp holds 32 / G consecutive points of one lobe (G = 1 unless SPLIT);
+// consecutive warps cycle through the lobes of the same points.
+template <bool STATS, int FLAGS, bool SPLIT>
 __global__ void __launch_bounds__(BAKE_THREADS, FIPT_BAKE_MINB)
 k_bake(SceneView sc, const fipt_query* __restrict__ q, int64_t N, BakeArgs A,
        float* __restrict__ Ld, float* __restrict__ Ls0, float* __restrict__ Ls1, int32_t* status,
-       unsigned long long* stats, const int32_t* __restrict__ order) {
+       unsigned long long* stats, const int32_t* __restrict__ order, int log_g) {
     const int L = 1 + A.K;
     const int64_t g = blockIdx.x * (int64_t)BAKE_THREADS + threadIdx.x;
     const int64_t w = g >> 5;
     const int lane = (int)(g & 31);
     const int lobe = (int)(w % L);
-    const int64_t p = (w / L) * 32 + lane;
-    if ((w / L) * 32 >= N) return;          // whole warp past the end
+    const int64_t p0 = SPLIT ? (w / L) << (5 - log_g) : (w / L) * 32;
+    const int64_t p = p0 + (SPLIT ? lane >> log_g : lane);
+    if (p0 >= N) return;                    // whole warp past the end
     bool valid = p < N;
     int64_t pq = p;                         // the query this slot bakes
     if (order && valid) {
@@ -390,7 +405,7 @@ k_bake(SceneView sc, const fipt_query* __restrict__ q, int64_t N, BakeArgs A,
             pq = 0;
         }
     }
-    bake_item<STATS, FLAGS>(sc, q, pq, lobe, valid, A, Ld, Ls0, Ls1, status, stats);
+    bake_item<STATS, FLAGS, SPLIT>(sc, q, pq, lobe, valid, A, Ld, Ls0, Ls1, status, stats, 1 << log_g);
 }
 
 // ---------------------------------------------------------------- device-resident serving loop
@@ -565,7 +580,7 @@ k_serve_bake(const BakeChunk* __restrict__ chunks, ServeShared* sh, ServeCounter
         const int64_t p = (wl / L) * 32 + lane;
         const bool valid = p < C.n;
         const int64_t pq = (C.order && valid) ? (int64_t)C.order[p] : p;
-        bake_item<false, FLAGS>(C.sc, C.q, pq, lobe, valid, C.A, C.Ld, C.Ls0, C.Ls1, status, nullptr);
+        bake_item<false, FLAGS, false>(C.sc, C.q, pq, lobe, valid, C.A, C.Ld, C.Ls0, C.Ls1, status, nullptr);
         __syncwarp();
         if (lane == 0) {
             __threadfence();
@@ -805,6 +820,34 @@ extern "C" fipt_status fipt_query_order(fipt_scene* s, const fipt_query* q, int6
     return FIPT_OK;
 }
 
+namespace {
+// log2 of the lanes that share a (point, lobe) pair, from how many times the
+// pairs, a lane each, would fill the GPU's warp slots.  Few pairs leave most
+// of the chip idle and end in a long tail, and lanes on one point and
+// neighbouring cells of directions also walk more alike than lanes on
+// neighbouring points that are far apart; with many pairs the points of a
+// warp lie close together and the unsplit warp is the coherent one.
+// Measured, ms for 1 / 2 / 4 / 8 / 16 / 32 lanes per pair (fills):
+//   room, 3,001 points x 64 (0.07)        4.40  2.17  1.38  0.92  0.69  0.63
+//   room, 20,011 x 64 (0.45)              5.81  3.76  2.90  2.54  2.41  2.63
+//   floor, 100,003 x 64 (2.3)            14.9  11.8  10.6  10.3  10.5  12.1
+//   room, 2^18 x 64 (5.9)                29.3  26.1  25.5  26.5  27.6  31.7
+//   floor, 2^19 x 64 (11.8)              50.9  47.2  46.6  49.2  52.3  61.4
+//   room, 2^20 x 128 (23.6)               191   185   189   200   206   229
+//   floor, 2^22 x 64 (94)                 333   335   349   381   411   488
+// A small tree's walks are short, and the shared adding up weighs three times
+// as much: Cornell box, 36 triangles,
+//   4,096 x 64 (0.09)                    0.84  0.48  0.33  0.30  0.30  0.36
+//   20,011 x 64 (0.45)                   1.14  0.91  0.82  0.79  0.86  1.20
+//   1,000,003 x 32 with a sky (16.1)     16.2  16.8  17.2  18.8  23.1  36.7
+int bake_split(int64_t pairs, int64_t T, int least_spp, int sms) {
+    const double fills = (double)pairs / (2048.0 * sms) * (T < 4096 ? 3.0 : 1.0);
+    int g = fills < 0.1 ? 5 : fills < 1.0 ? 4 : fills < 3.0 ? 3 : fills < 12.0 ? 2 : fills < 60.0 ? 1 : 0;
+    while ((1 << g) > least_spp) --g;             // no lane without a sample
+    return g;
+}
+}  // namespace
+
 extern "C" fipt_status fipt_bake(fipt_scene* s, const fipt_query* q, int64_t N,
                                  const fipt_bake_params* prm, float* Ld, float* Ls0, float* Ls1,
                                  fipt_stream stream) {
@@ -830,16 +873,27 @@ extern "C" fipt_status fipt_bake(fipt_scene* s, const fipt_query* q, int64_t N,
     A.K = prm->K;
     set_strata(A);
     for (int k = 0; k < FIPT_MAX_K; ++k) A.sigma[k] = k < prm->K ? prm->sigma[k] : 1.0f;
-    const int64_t warps = ((N + 31) / 32) * (1 + prm->K);
+    int dev = 0, sms = 0;
+    FIPT_CUDA(cudaGetDevice(&dev));
+    FIPT_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const int log_g = bake_split(N * (1 + prm->K), s->T, std::min(prm->spp_diffuse, prm->spp_specular), sms);
+    const int64_t per_warp = 32 >> log_g;
+    const int64_t warps = ((N + per_warp - 1) / per_warp) * (1 + prm->K);
     const int64_t threads = warps * 32;
     const unsigned nb = blocks(threads, BAKE_THREADS);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int flags = (s->env ? 1 : 0) | (s->vox ? 2 : 0);
     const SceneView sv = s->view();
     unsigned long long* stats = prm->stats;
-#define FIPT_BAKE_CASE(ST, FL)                                                                   \
-    FIPT_LAUNCH((k_bake<ST, FL>), nb, BAKE_THREADS, 0, st, sv, q, N, A, Ld, Ls0, Ls1, s->ctx->status, \
-                stats, prm->order)
+#define FIPT_BAKE_CASE(ST, FL)                                                                                    \
+    do {                                                                                                          \
+        if (log_g)                                                                                                \
+            FIPT_LAUNCH((k_bake<ST, FL, true>), nb, BAKE_THREADS, 0, st, sv, q, N, A, Ld, Ls0, Ls1, s->ctx->status, \
+                        stats, prm->order, log_g);                                                                \
+        else                                                                                                      \
+            FIPT_LAUNCH((k_bake<ST, FL, false>), nb, BAKE_THREADS, 0, st, sv, q, N, A, Ld, Ls0, Ls1,              \
+                        s->ctx->status, stats, prm->order, 0);                                                    \
+    } while (0)
     if (stats) {
         switch (flags) {
             case 0: FIPT_BAKE_CASE(true, 0); break;
