@@ -12,7 +12,7 @@
 namespace {
 
 constexpr int SORT_THREADS = 256;
-constexpr int SORT_ITEMS = 8;
+constexpr int SORT_ITEMS = 8;             // keys per thread (16 measured the same for 8-byte pairs)
 constexpr int SORT_TILE = SORT_THREADS * SORT_ITEMS;
 constexpr int RADIX = 256;
 constexpr int SCAN_THREADS = 1024;
@@ -123,59 +123,173 @@ k_scan_apply(uint32_t* __restrict__ a, int64_t m, const uint32_t* __restrict__ b
     }
 }
 
-// Stable scatter: an element's rank among equal digits in its tile follows
-// (iteration, warp, lane), i.e. index order.
+// The stable order of a block's keys by one digit.  A warp holds 32 * ITEMS
+// consecutive keys, key r of lane l at r * 32 + l, and ranks them against its
+// own counters without the rest of the block; then 256 threads turn the warps'
+// counters into offsets and scan the digits' totals.
+template <int THREADS, int ITEMS>
+struct DigitRank {
+    static constexpr int WARPS = THREADS / 32;
+    uint32_t cnt[WARPS][RADIX];    // keys with the digit in earlier warps
+    uint32_t start[RADIX];         // keys with a smaller digit
+    uint32_t wsum[RADIX / 32];
+
+    // digit[r]: RADIX for no key.  pos[r]: the key's place in the block's order.
+    __device__ __forceinline__ void order(const uint32_t (&digit)[ITEMS], uint32_t (&pos)[ITEMS]) {
+        constexpr unsigned FULL = 0xffffffffu;
+        const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+        for (int i = tid; i < WARPS * RADIX; i += THREADS) (&cnt[0][0])[i] = 0;
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < ITEMS; ++r) {
+            const uint32_t d = digit[r];
+            const unsigned same = __match_any_sync(FULL, d);
+            const uint32_t before = d < RADIX ? cnt[warp][d] : 0u;
+            pos[r] = before + __popc(same & ((1u << lane) - 1u));
+            __syncwarp();
+            if (d < RADIX && lane == __ffs(same) - 1) cnt[warp][d] = before + __popc(same);
+            __syncwarp();
+        }
+        __syncthreads();
+        uint32_t total = 0, incl = 0;
+        if (tid < RADIX) {
+#pragma unroll
+            for (int w = 0; w < WARPS; ++w) {
+                const uint32_t c = cnt[w][tid];
+                cnt[w][tid] = total;
+                total += c;
+            }
+            incl = total;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(FULL, incl, o);
+                if (lane >= o) incl += y;
+            }
+            if (lane == 31) wsum[warp] = incl;
+        }
+        __syncthreads();
+        if (tid < RADIX) {
+            uint32_t s = incl - total;
+            for (int w = 0; w < warp; ++w) s += wsum[w];
+            start[tid] = s;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < ITEMS; ++r)
+            if (digit[r] < RADIX) pos[r] += start[digit[r]] + cnt[warp][digit[r]];
+    }
+};
+
+// Stable scatter of a tile: its pairs are put in digit order in shared
+// memory and written from there, so that a digit's run leaves in consecutive
+// addresses.  Bound by the ranking's matches, then by those writes: 2,045,464
+// pairs of 12 bytes 31.8 -> 23.3 us a pass, 4,194,304 of 8 bytes 26.6 as before
+// (ranking 256 keys at a time with four block barriers each, and writing every
+// pair to its place directly, before).
 template <class K>
-__global__ void __launch_bounds__(SORT_THREADS)
+__global__ void __launch_bounds__(SORT_THREADS, 4)
 k_sort_scatter(const K* __restrict__ kin, const uint32_t* __restrict__ vin, K* __restrict__ kout,
                uint32_t* __restrict__ vout, int64_t n, const uint32_t* __restrict__ n_dev, int shift,
                const uint32_t* __restrict__ hist) {
+    constexpr int ITEMS = SORT_ITEMS, TILE = SORT_TILE;
     if (n_dev && (int64_t)*n_dev < n) n = *n_dev;
-    if ((int64_t)blockIdx.x * SORT_TILE >= n) return;   // the whole tile is past the keys
-    constexpr int WARPS = SORT_THREADS / 32;
-    __shared__ uint32_t base_off[RADIX];
-    __shared__ uint32_t run[RADIX];
-    __shared__ uint32_t wcnt[WARPS][RADIX];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    base_off[tid] = hist[(int64_t)tid * gridDim.x + blockIdx.x];
-    run[tid] = 0;
-    const uint32_t lt_mask = (1u << lane) - 1u;
-    const int64_t base = (int64_t)blockIdx.x * SORT_TILE;
-    for (int it = 0; it < SORT_ITEMS; ++it) {
-        const int64_t i = base + it * SORT_THREADS + tid;
-        const bool valid = i < n;
-        K k = 0;
-        uint32_t v = 0;
-        uint32_t digit = RADIX;
-        if (valid) {
-            k = kin[i];
-            v = vin[i];
-            digit = (uint32_t)(k >> shift) & (RADIX - 1);
+    const int64_t base = (int64_t)blockIdx.x * TILE;
+    if (base >= n) return;                                  // the whole tile is past the keys
+    __shared__ DigitRank<SORT_THREADS, ITEMS> rank;
+    __shared__ K sk[TILE];
+    __shared__ uint32_t sv[TILE];
+    __shared__ uint32_t to[RADIX];                          // a digit's first place minus its place in the tile
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int64_t first = base + (tid >> 5) * (32 * ITEMS) + lane;
+    K k[ITEMS];
+    uint32_t v[ITEMS], digit[ITEMS], pos[ITEMS];
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+        const int64_t i = first + 32 * r;
+        digit[r] = RADIX;
+        if (i < n) {
+            k[r] = kin[i];
+            v[r] = vin[i];
+            digit[r] = (uint32_t)(k[r] >> shift) & (RADIX - 1);
         }
+    }
+    rank.order(digit, pos);
+    if (tid < RADIX) to[tid] = hist[(int64_t)tid * gridDim.x + blockIdx.x] - rank.start[tid];
 #pragma unroll
-        for (int w = 0; w < WARPS; ++w) wcnt[w][tid] = 0;
-        __syncthreads();
-        const uint32_t peers = __match_any_sync(0xffffffffu, digit);
-        const uint32_t rank = __popc(peers & lt_mask);
-        if (valid && rank == 0) wcnt[warp][digit] = __popc(peers);
-        __syncthreads();
-        {
-            uint32_t r = run[tid];
+    for (int r = 0; r < ITEMS; ++r)
+        if (digit[r] < RADIX) {
+            sk[pos[r]] = k[r];
+            sv[pos[r]] = v[r];
+        }
+    __syncthreads();
+    const int here = (int)(n - base < TILE ? n - base : TILE);
 #pragma unroll
-            for (int w = 0; w < WARPS; ++w) {
-                const uint32_t c = wcnt[w][tid];
-                wcnt[w][tid] = r;
-                r += c;
+    for (int r = 0; r < ITEMS; ++r) {
+        const int i = r * SORT_THREADS + tid;
+        if (i < here) {
+            const K key = sk[i];
+            const uint32_t at = to[(uint32_t)(key >> shift) & (RADIX - 1)] + (uint32_t)i;
+            kout[at] = key;
+            vout[at] = sv[i];
+        }
+    }
+}
+
+// All passes of a small sort in one block, in place: the pairs stay in
+// registers between the passes and change places through shared memory.  It
+// replaces three launches a pass: four passes over 4,096 keys of 32 bits, 75 us
+// and the gaps of twelve launches -> 20 us.  One block holds 8,192 pairs.
+constexpr int SMALL_THREADS = 1024;
+constexpr int64_t SMALL_MAX = SMALL_THREADS * 8;
+
+template <class K, int SMALL_ITEMS>
+struct SmallSort {
+    DigitRank<SMALL_THREADS, SMALL_ITEMS> rank;
+    K k[SMALL_THREADS * SMALL_ITEMS];
+    uint32_t v[SMALL_THREADS * SMALL_ITEMS];
+};
+
+template <class K, int SMALL_ITEMS>
+__global__ void __launch_bounds__(SMALL_THREADS)
+k_sort_small(K* __restrict__ keys, uint32_t* __restrict__ vals, int n, const uint32_t* __restrict__ n_dev, int bits) {
+    extern __shared__ __align__(16) unsigned char small_mem[];
+    SmallSort<K, SMALL_ITEMS>& sm = *reinterpret_cast<SmallSort<K, SMALL_ITEMS>*>(small_mem);
+    if (n_dev && *n_dev < (uint32_t)n) n = (int)*n_dev;
+    const int first = (threadIdx.x >> 5) * (32 * SMALL_ITEMS) + (threadIdx.x & 31);
+    K k[SMALL_ITEMS];
+    uint32_t v[SMALL_ITEMS], digit[SMALL_ITEMS], pos[SMALL_ITEMS];
+#pragma unroll
+    for (int r = 0; r < SMALL_ITEMS; ++r) {
+        const int i = first + 32 * r;
+        k[r] = i < n ? keys[i] : 0;
+        v[r] = i < n ? vals[i] : 0;
+    }
+    for (int shift = 0; shift < bits; shift += 8) {
+#pragma unroll
+        for (int r = 0; r < SMALL_ITEMS; ++r)
+            digit[r] = first + 32 * r < n ? (uint32_t)(k[r] >> shift) & (RADIX - 1) : RADIX;
+        sm.rank.order(digit, pos);
+#pragma unroll
+        for (int r = 0; r < SMALL_ITEMS; ++r)
+            if (digit[r] < RADIX) {
+                sm.k[pos[r]] = k[r];
+                sm.v[pos[r]] = v[r];
             }
-            run[tid] = r;
-        }
         __syncthreads();
-        if (valid) {
-            const uint32_t pos = base_off[digit] + wcnt[warp][digit] + rank;
-            kout[pos] = k;
-            vout[pos] = v;
+#pragma unroll
+        for (int r = 0; r < SMALL_ITEMS; ++r)
+            if (first + 32 * r < n) {
+                k[r] = sm.k[first + 32 * r];
+                v[r] = sm.v[first + 32 * r];
+            }
+    }
+#pragma unroll
+    for (int r = 0; r < SMALL_ITEMS; ++r) {
+        const int i = first + 32 * r;
+        if (i < n) {
+            keys[i] = k[r];
+            vals[i] = v[r];
         }
-        __syncthreads();
     }
 }
 
@@ -910,6 +1024,15 @@ static fipt_status scan_hist(uint32_t* hist, int64_t m, uint32_t* bsum, cudaStre
     return FIPT_OK;
 }
 
+template <class K, int ITEMS>
+static fipt_status sort_small(K* keys, uint32_t* vals, int n, int bits, cudaStream_t st, const uint32_t* n_dev) {
+    constexpr size_t smem = sizeof(SmallSort<K, ITEMS>);
+    FIPT_CUDA(cudaFuncSetAttribute(k_sort_small<K, ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    FIPT_LAUNCH((k_sort_small<K, ITEMS>), 1, SMALL_THREADS, smem, st, keys, vals, n, n_dev, bits);
+    FIPT_LAUNCHED("small radix sort");
+    return FIPT_OK;
+}
+
 template <class K>
 fipt_status radix_sort_pairs(K* keys, K* keys_alt, uint32_t* vals, uint32_t* vals_alt,
                              uint32_t* hist, int64_t n, int bits, cudaStream_t st, K** out_keys,
@@ -917,7 +1040,12 @@ fipt_status radix_sort_pairs(K* keys, K* keys_alt, uint32_t* vals, uint32_t* val
     K *ka = keys, *kb = keys_alt;
     uint32_t *va = vals, *vb = vals_alt;
     const int64_t nb = sort_blocks(n);
-    if (n > 0) {
+    if (n > 0 && n <= SMALL_MAX) {
+        fipt_status r = n <= 2 * SMALL_THREADS   ? sort_small<K, 2>(keys, vals, (int)n, bits, st, n_dev)
+                        : n <= 4 * SMALL_THREADS ? sort_small<K, 4>(keys, vals, (int)n, bits, st, n_dev)
+                                                 : sort_small<K, 8>(keys, vals, (int)n, bits, st, n_dev);
+        if (r != FIPT_OK) return r;
+    } else if (n > 0) {
         for (int shift = 0; shift < bits; shift += 8) {
             FIPT_LAUNCH(k_sort_hist<K>, (unsigned)nb, SORT_THREADS, 0, st, ka, n, n_dev, shift, hist);
             fipt_status r = scan_hist(hist, (int64_t)RADIX * nb, hist + hist_words(n), st);
