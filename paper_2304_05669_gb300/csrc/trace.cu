@@ -29,16 +29,24 @@ k_trace(SceneView sc, const float* __restrict__ orig, const float* __restrict__ 
     hit_front[i] = b.any() && b.front() ? 1 : 0;
 }
 
+// A warp looks through a tile of 8 x 4 pixels (2^log_tw x 32 / 2^log_tw),
+// whose rays walk the tree more alike than those of 32 pixels of a row (24
+// views of 640 x 416 in the room: 820 -> 776 us).  Lanes past the image's
+// edges have no ray.
 __global__ void __launch_bounds__(TRACE_THREADS)
-k_camera(SceneView sc, const float* __restrict__ cams, int W, int H, int64_t P,
+k_camera(SceneView sc, const float* __restrict__ cams, int W, int H, int log_tw, int tiles_x, int tiles_y, int64_t tiles,
          fipt_query* __restrict__ out, int32_t* __restrict__ valid, int32_t* status) {
-    const int64_t slot = blockIdx.x * (int64_t)TRACE_THREADS + threadIdx.x;
-    const bool on = slot < P;
-    const int64_t p = on ? slot : P - 1;
-    const int64_t wh = (int64_t)W * H;
-    const int v = (int)(p / wh);
-    const int64_t rem = p - v * wh;
-    const int j = (int)(rem / W), i = (int)(rem - (int64_t)j * W);
+    const int64_t tile = (blockIdx.x * (int64_t)TRACE_THREADS + threadIdx.x) >> 5;
+    if (tile >= tiles) return;                             // whole warp
+    const int lane = threadIdx.x & 31;
+    const int64_t row = tile / tiles_x;                    // tile rows, view after view
+    const int v = (int)(row / tiles_y);
+    int i = ((int)(tile - row * tiles_x) << log_tw) + (lane & ((1 << log_tw) - 1));
+    int j = ((int)(row - (int64_t)v * tiles_y) << (5 - log_tw)) + (lane >> log_tw);
+    const bool on = i < W && j < H;
+    i = min(i, W - 1);
+    j = min(j, H - 1);
+    const int64_t p = ((int64_t)v * H + j) * W + i;
     const float* c = cams + 10 * v;
     float fx = c[3], fy = c[4], fz = c[5];
     const float fl = 1.0f / sqrtf(fx * fx + fy * fy + fz * fz);
@@ -140,27 +148,40 @@ __global__ void __launch_bounds__(1024) k_scan_bsum(uint32_t* __restrict__ a, in
     if (threadIdx.x == 0) *n_out = (int64_t)carry < max_out ? (int64_t)carry : max_out;
 }
 
+// A block lists the sources of its valid records in shared memory, then its
+// threads copy them as one stream of 8-byte words (a record is five), so both
+// the reads and the writes are contiguous: 6,389,760 records, half of them
+// kept, 258 -> 48 us (a thread copying its own eight records before).
+// Blocks past max_out leave at once.
 __global__ void __launch_bounds__(CMP_THREADS)
 k_compact(const fipt_query* __restrict__ in, const int32_t* __restrict__ valid, int64_t P,
           int64_t max_out, const uint32_t* __restrict__ boff, fipt_query* __restrict__ out,
           int32_t* __restrict__ pixel_of) {
     __shared__ uint32_t ws[32];
-    const int64_t base = (int64_t)blockIdx.x * CMP_TILE + threadIdx.x * CMP_ITEMS;
-    uint32_t c = 0;
+    __shared__ uint16_t src[CMP_TILE];
+    const int64_t pos0 = boff[blockIdx.x];
+    if (pos0 >= max_out) return;
+    const int64_t tile = (int64_t)blockIdx.x * CMP_TILE, base = tile + threadIdx.x * CMP_ITEMS;
+    uint32_t keep = 0;
 #pragma unroll
-    for (int k = 0; k < CMP_ITEMS; ++k) c += (base + k < P && valid[base + k] != 0) ? 1u : 0u;
+    for (int k = 0; k < CMP_ITEMS; ++k) keep |= (base + k < P && valid[base + k] != 0) ? 1u << k : 0u;
     uint32_t tot;
-    int64_t pos = (int64_t)boff[blockIdx.x] + block_exclusive_scan(c, ws, &tot);
-    for (int k = 0; k < CMP_ITEMS; ++k) {
-        const int64_t i = base + k;
-        if (i < P && valid[i] != 0) {
-            if (pos < max_out) {
-                out[pos] = in[i];
-                if (pixel_of) pixel_of[pos] = (int32_t)i;
-            }
-            ++pos;
-        }
+    uint32_t at = block_exclusive_scan((uint32_t)__popc(keep), ws, &tot);
+#pragma unroll
+    for (int k = 0; k < CMP_ITEMS; ++k)
+        if (keep >> k & 1) src[at++] = (uint16_t)(threadIdx.x * CMP_ITEMS + k);
+    __syncthreads();
+    const int n = (int)(max_out - pos0 < tot ? max_out - pos0 : tot);
+    static_assert(sizeof(fipt_query) == 40, "five 8-byte words");
+    const float2* from = reinterpret_cast<const float2*>(in + tile);
+    float2* to = reinterpret_cast<float2*>(out + pos0);
+#pragma unroll 4
+    for (int w = threadIdx.x; w < 5 * n; w += CMP_THREADS) {
+        const int rec = w / 5;
+        to[w] = __ldg(from + 5 * src[rec] + (w - 5 * rec));
     }
+    if (pixel_of)
+        for (int k = threadIdx.x; k < n; k += CMP_THREADS) pixel_of[pos0 + k] = (int32_t)(tile + src[k]);
 }
 
 // ---------------------------------------------------------------- bake
@@ -734,7 +755,14 @@ extern "C" fipt_status fipt_camera_queries(fipt_scene* s, const float* cams, int
     FIPT_REQUIRE(fipt_aligned(cams, 4) && fipt_aligned(out, 16) && fipt_aligned(valid, 4),
                  "cams 4-byte, out 16-byte, valid 4-byte alignment required");
     FIPT_CUDA(cudaSetDevice(s->ctx->device));
-    FIPT_LAUNCH(k_camera, blocks(P, TRACE_THREADS), TRACE_THREADS, 0, static_cast<cudaStream_t>(stream), s->view(), cams, W, H, P, out, valid, s->ctx->status);
+    int log_tw = 3;                       // narrower or wider tiles for images under 8 pixels across or 4 down
+    while ((1 << log_tw) > W) --log_tw;
+    while (log_tw < 5 && (32 >> log_tw) > H) ++log_tw;
+    const int tw = 1 << log_tw, th = 32 >> log_tw;
+    const int tiles_x = (int)(((int64_t)W + tw - 1) / tw), tiles_y = (int)(((int64_t)H + th - 1) / th);
+    const int64_t tiles = (int64_t)nViews * tiles_x * tiles_y;
+    FIPT_LAUNCH(k_camera, blocks(tiles * 32, TRACE_THREADS), TRACE_THREADS, 0, static_cast<cudaStream_t>(stream),
+                s->view(), cams, W, H, log_tw, tiles_x, tiles_y, tiles, out, valid, s->ctx->status);
     FIPT_LAUNCHED("camera_queries");
     return FIPT_OK;
 }
