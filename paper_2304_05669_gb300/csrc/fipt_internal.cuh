@@ -24,6 +24,7 @@ struct SceneConst {
     float eps;          // ray-origin offset, 1e-4 * largest extent
     int n_emit;         // emitter triangles (any L_e channel > 0)
     double A_emit;      // their total area
+    double morton_scale[3];   // Morton cells per unit length along each axis (0: a flat axis)
 };
 
 // Internal BVH node (64 bytes): both child boxes plus child references.

@@ -340,6 +340,10 @@ __global__ void k_bounds_final(SceneConst* c, int64_t nV) {
         c->lo[a] = nV ? ordered_to_float(c->lo_key[a]) : 0.0f;
         c->hi[a] = nV ? ordered_to_float(c->hi_key[a]) : 0.0f;
         ext = fmaxf(ext, c->hi[a] - c->lo[a]);
+        // cells per unit length of the Morton grid, divided once here and not per triangle (FP64 runs at 1/64
+        // of the float32 rate: 254 -> 140 us for the codes of 2,045,464 triangles)
+        const double e = __dsub_rn((double)c->hi[a], (double)c->lo[a]);
+        c->morton_scale[a] = e > 0.0 ? __ddiv_rn(2097152.0, e) : 0.0;
     }
     c->eps = 1e-4f * ext;
 }
@@ -380,14 +384,12 @@ __global__ void k_morton(const float* __restrict__ V, int64_t nV, const int32_t*
         const float x0 = V[3 * i0 + a], x1 = V[3 * i1 + a], x2 = V[3 * i2 + a];
         const float mn = fminf(fminf(x0, x1), x2), mx = fmaxf(fmaxf(x0, x1), x2);
         const double cc = __dmul_rn(0.5, __dadd_rn((double)mn, (double)mx));
-        const double lo = (double)c->lo[a];
-        const double ext = __dsub_rn((double)c->hi[a], lo);
-        if (!(ext > 0.0)) {
+        const double scale = c->morton_scale[a];
+        if (scale == 0.0) {                                // a flat axis
             q[a] = 0;
             continue;
         }
-        const double scale = __ddiv_rn(2097152.0, ext);
-        double f = floor(__dmul_rn(__dsub_rn(cc, lo), scale));
+        double f = floor(__dmul_rn(__dsub_rn(cc, (double)c->lo[a]), scale));
         f = f < 0.0 ? 0.0 : (f > 2097151.0 ? 2097151.0 : f);
         q[a] = (uint32_t)f;
     }
@@ -678,7 +680,12 @@ __device__ __forceinline__ void better_part(float& v, int& P, int lane_mask) {
 // 2,045,464 triangles: 7.4 -> 1.9 ms (with each lane forming the whole
 // treelet in local arrays, the partitions of a subset on one lane and lane 0
 // alone writing), the same trees.
-__device__ void restructure_warp(BvhNode* nodes, int32_t* parent, int32_t* leaf_parent, int p,
+//
+// A record's d.z holds the pass that last rewrote it.  A treelet none of whose
+// records was rewritten in the last pass or so far in this one is the treelet
+// the last pass found at p and kept, so this pass would keep it too and leaves
+// it: three passes over the floor 5.8 -> 5.1 ms.
+__device__ void restructure_warp(BvhNode* nodes, int32_t* parent, int32_t* leaf_parent, int p, int pass,
                                  TreeletTables& tb, const uint8_t* subsets, int lane) {
     constexpr unsigned FULL = 0xffffffffu;
     // lane 0 and 1: p's children
@@ -686,11 +693,14 @@ __device__ void restructure_warp(BvhNode* nodes, int32_t* parent, int32_t* leaf_
     Box box = Box{0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
     float area = 0.0f;
     int inner = p;                                         // lane k: the treelet's internal node k
+    bool fresh = false;                                    // rewritten in the last pass or this one
     const auto take_child = [&](int n, bool second) {      // the lane's leaf becomes a child of n
         const float4* q = reinterpret_cast<const float4*>(nodes + n);
         const float4 a = __ldcg(q + (second ? 1 : 0));
         const float2 z = __ldcg(reinterpret_cast<const float2*>(q + 2) + (second ? 1 : 0));
-        ref = __ldcg(reinterpret_cast<const int*>(q + 3) + (second ? 1 : 0));
+        const int4 d = __ldcg(reinterpret_cast<const int4*>(q + 3));
+        ref = second ? d.y : d.x;
+        fresh = fresh || d.z >= pass - 1;
         box = Box{a.x, a.y, z.x, a.z, a.w, z.y};
         area = half_area(box);
     };
@@ -713,6 +723,7 @@ __device__ void restructure_warp(BvhNode* nodes, int32_t* parent, int32_t* leaf_
         ++m;
     }
     if (m < 3) return;                                     // two leaves have one topology (uniform)
+    if (!__any_sync(FULL, fresh)) return;
     if (lane < m) tb.box[lane] = box;
     __syncwarp();
     const int full = (1 << m) - 1;
@@ -825,7 +836,7 @@ __device__ void restructure_warp(BvhNode* nodes, int32_t* parent, int32_t* leaf_
         __stcg(q + 0, make_float4(b[0].lx, b[0].ly, b[0].hx, b[0].hy));
         __stcg(q + 1, make_float4(b[1].lx, b[1].ly, b[1].hx, b[1].hy));
         __stcg(q + 2, make_float4(b[0].lz, b[0].hz, b[1].lz, b[1].hz));
-        __stcg(reinterpret_cast<int4*>(q + 3), make_int4(r0, r1, 0, 0));
+        __stcg(reinterpret_cast<int4*>(q + 3), make_int4(r0, r1, pass, 0));
         __stcg(r0 >= 0 ? parent + r0 : leaf_parent + ~r0, inner);
         __stcg(r1 >= 0 ? parent + r1 : leaf_parent + ~r1, inner);
         __threadfence();
@@ -839,13 +850,14 @@ constexpr int TL_THREADS = 128;
 // its leaf; at every round the warp restructures, one after the other, the
 // nodes its lanes were second to reach.  A climb longer than any valid
 // tree allows (a corrupt parent chain) stops and raises the step flag.
-__global__ void __launch_bounds__(TL_THREADS)
-k_treelets(BvhNode* nodes, int32_t* parent, int32_t* leaf_parent, int32_t* flags, int64_t T, int32_t* status) {
+__global__ void __launch_bounds__(TL_THREADS, 10)
+k_treelets(BvhNode* nodes, int32_t* parent, int32_t* leaf_parent, int32_t* flags, int64_t T, int pass,
+           int32_t* status) {
     constexpr unsigned FULL = 0xffffffffu;
     __shared__ TreeletTables tabs[TL_THREADS / 32];
     __shared__ uint8_t subsets[sizeof(SubsetTable)];
     TreeletTables& tb = tabs[threadIdx.x >> 5];
-    if (threadIdx.x < sizeof(SubsetTable)) subsets[threadIdx.x] = c_subsets.s[threadIdx.x];
+    for (int i = threadIdx.x; i < (int)sizeof(SubsetTable); i += TL_THREADS) subsets[i] = c_subsets.s[i];
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const int64_t leaf = blockIdx.x * (int64_t)TL_THREADS + threadIdx.x;
@@ -874,7 +886,7 @@ k_treelets(BvhNode* nodes, int32_t* parent, int32_t* leaf_parent, int32_t* flags
         while (todo) {
             const int l = __ffs(todo) - 1;
             todo &= todo - 1;
-            restructure_warp(nodes, parent, leaf_parent, __shfl_sync(FULL, p, l), tb, subsets, lane);
+            restructure_warp(nodes, parent, leaf_parent, __shfl_sync(FULL, p, l), pass, tb, subsets, lane);
         }
         if (act) {
             __threadfence();
@@ -1214,7 +1226,7 @@ extern "C" fipt_status fipt_scene_optimize(fipt_scene* s, int32_t passes, fipt_s
     for (int k = 0; k < passes; ++k) {
         FIPT_CUDA(cudaMemsetAsync(s->flags, 0, sizeof(int32_t) * (size_t)(T - 1), st));
         FIPT_LAUNCH(k_treelets, grid_for(T, TL_THREADS), TL_THREADS, 0, st, s->nodes, s->parent, s->leaf_parent, s->flags, T,
-                    s->ctx->status);
+                    k + 1, s->ctx->status);
     }
     FIPT_LAUNCHED("treelet restructuring");
     s->restructured = true;
