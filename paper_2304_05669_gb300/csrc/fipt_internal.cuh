@@ -142,7 +142,8 @@ struct alignas(256) BakeChunk {
     float *Ld, *Ls0, *Ls1;   // the chunk's first output rows (the request's first, with an order)
     const int32_t* order;    // NULL, or the chunk's slots of the request's order: slot p bakes query order[p]
     int64_t n;               // points in the chunk
-    int64_t warp_begin;      // first global warp of the chunk
+    int64_t warp_begin;      // first global warp item of the chunk
+    int log_g;               // log2 of the lanes that share a pair (bake_split of the request)
     BakeArgs A;              // A.point_base = request-local index of the first point
 };
 
@@ -186,6 +187,15 @@ struct ServeCounters {
     int quit_r;                // nonzero: a render warp found no work for long; the render launch leaves
     int pad;
 };
+
+// log2 of the lanes that share each of `pairs` (point, lobe) pairs of a bake in
+// a scene of T triangles, on the current device; at most one lane a sample.
+int bake_split(int64_t pairs, int64_t T, int least_spp);
+// Warp items of n points and L lobes at that split.
+__host__ __device__ inline int64_t bake_warps(int64_t n, int L, int log_g) {
+    const int64_t per = 32 >> log_g;
+    return (n + per - 1) / per * L;
+}
 
 // The server's resident bake loop (see k_serve_bake) and render loop (see
 // k_serve_render).

@@ -575,10 +575,12 @@ void fipt_server::stage_chunks() {
         Req* q = reqs[t];
         const fipt_bake_params& P = q->r.params;
         const int64_t rpp = rays_per_point(P);
+        const int log_g = bake_split(q->r.n * (1 + P.K), scenes[q->r.target]->T,
+                                     std::min(P.spp_diffuse, P.spp_specular));
         int64_t got = 0;
         while (q->next < q->r.n && n_staged < kQueue) {
             const int64_t c = std::min<int64_t>(chunk_points, q->r.n - q->next);
-            const int64_t items = ((c + 31) / 32) * (1 + P.K);
+            const int64_t items = bake_warps(c, 1 + P.K, log_g);
             const bool full = items_ahead + items > lookahead_items && rays_ahead + c * rpp > lookahead_rays;
             if (items_ahead > 0 && (full || got + items > share)) break;
             BakeChunk& C = q_host[n_staged];
@@ -599,6 +601,7 @@ void fipt_server::stage_chunks() {
             }
             C.n = c;
             C.warp_begin = warps_staged;
+            C.log_g = log_g;
             C.A.key = make_uint2((uint32_t)P.seed, (uint32_t)(P.seed >> 32));
             C.A.request_id = P.request_id;
             C.A.point_base = q->order_off >= 0 ? 0u : (uint32_t)q->next;

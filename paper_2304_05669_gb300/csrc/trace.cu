@@ -598,14 +598,16 @@ k_serve_bake(const BakeChunk* __restrict__ chunks, ServeShared* sh, ServeCounter
         const int L = 1 + C.A.K;
         const int64_t wl = w - C.warp_begin;
         const int lobe = (int)(wl % L);
-        const int64_t p = (wl / L) * 32 + lane;
+        const int log_g = C.log_g;
+        const int64_t p = ((wl / L) << (5 - log_g)) + (lane >> log_g);
         const bool valid = p < C.n;
         const int64_t pq = (C.order && valid) ? (int64_t)C.order[p] : p;
-        bake_item<false, FLAGS, false>(C.sc, C.q, pq, lobe, valid, C.A, C.Ld, C.Ls0, C.Ls1, status, nullptr);
+        bake_item<false, FLAGS, true>(C.sc, C.q, pq, lobe, valid, C.A, C.Ld, C.Ls0, C.Ls1, status, nullptr,
+                                      1 << log_g);
         __syncwarp();
         if (lane == 0) {
             __threadfence();
-            const int items = (int)(((C.n + 31) / 32) * L);
+            const int items = (int)bake_warps(C.n, L, log_g);
             if (atomicAdd(done_count + ci, 1) == items - 1) {
                 __threadfence_system();
                 st_release_sys(done_flag + ci, 1);
@@ -848,7 +850,6 @@ extern "C" fipt_status fipt_query_order(fipt_scene* s, const fipt_query* q, int6
     return FIPT_OK;
 }
 
-namespace {
 // log2 of the lanes that share a (point, lobe) pair, from how many times the
 // pairs, a lane each, would fill the GPU's warp slots.  Few pairs leave most
 // of the chip idle and end in a long tail, and lanes on one point and
@@ -868,13 +869,16 @@ namespace {
 //   4,096 x 64 (0.09)                    0.84  0.48  0.33  0.30  0.30  0.36
 //   20,011 x 64 (0.45)                   1.14  0.91  0.82  0.79  0.86  1.20
 //   1,000,003 x 32 with a sky (16.1)     16.2  16.8  17.2  18.8  23.1  36.7
-int bake_split(int64_t pairs, int64_t T, int least_spp, int sms) {
+int bake_split(int64_t pairs, int64_t T, int least_spp) {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+        return 0;
     const double fills = (double)pairs / (2048.0 * sms) * (T < 4096 ? 3.0 : 1.0);
     int g = fills < 0.1 ? 5 : fills < 1.0 ? 4 : fills < 3.0 ? 3 : fills < 12.0 ? 2 : fills < 60.0 ? 1 : 0;
     while ((1 << g) > least_spp) --g;             // no lane without a sample
     return g;
 }
-}  // namespace
 
 extern "C" fipt_status fipt_bake(fipt_scene* s, const fipt_query* q, int64_t N,
                                  const fipt_bake_params* prm, float* Ld, float* Ls0, float* Ls1,
@@ -901,13 +905,8 @@ extern "C" fipt_status fipt_bake(fipt_scene* s, const fipt_query* q, int64_t N,
     A.K = prm->K;
     set_strata(A);
     for (int k = 0; k < FIPT_MAX_K; ++k) A.sigma[k] = k < prm->K ? prm->sigma[k] : 1.0f;
-    int dev = 0, sms = 0;
-    FIPT_CUDA(cudaGetDevice(&dev));
-    FIPT_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const int log_g = bake_split(N * (1 + prm->K), s->T, std::min(prm->spp_diffuse, prm->spp_specular), sms);
-    const int64_t per_warp = 32 >> log_g;
-    const int64_t warps = ((N + per_warp - 1) / per_warp) * (1 + prm->K);
-    const int64_t threads = warps * 32;
+    const int log_g = bake_split(N * (1 + prm->K), s->T, std::min(prm->spp_diffuse, prm->spp_specular));
+    const int64_t threads = 32 * bake_warps(N, 1 + prm->K, log_g);
     const unsigned nb = blocks(threads, BAKE_THREADS);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int flags = (s->env ? 1 : 0) | (s->vox ? 2 : 0);
