@@ -399,18 +399,29 @@ __device__ __forceinline__ void node_test(const TraceRay& r, const BvhNode& n, f
 }
 
 // A node's record in two 32-byte loads (sm_100's widest), one per sector:
-// half the load instructions and fewer L1 wavefronts (79 -> 72 % of the data
-// pipe's peak on the room) than four 16-byte loads.  Records are 64-byte
-// aligned: the node arrays start 256-byte aligned in the scene's workspace.
+// half the load instructions of four 16-byte loads.  L1 returns 128 bytes a
+// cycle, so a warp's node costs it up to 16 cycles, about what issuing the
+// slab tests costs; SLIM leaves out the record's last 8 bytes (14 cycles) for
+// one more instruction, which pays where L1 is the bound (incoherent rays:
+// refinement of the room 40.4 -> 39.7 ms, the floor 41.2 -> 39.9) and not where
+// issue is (the room's bake 25.5 -> 25.7).  Records are 64-byte aligned: the
+// node arrays start 256-byte aligned in the scene's workspace.
+template <bool SLIM>
 __device__ __forceinline__ BvhNode load_node(const BvhNode* nodes, int i) {
     const BvhNode* p = nodes + i;
     BvhNode n;
     asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
         : "=f"(n.a.x), "=f"(n.a.y), "=f"(n.a.z), "=f"(n.a.w), "=f"(n.b.x), "=f"(n.b.y), "=f"(n.b.z), "=f"(n.b.w)
         : "l"(p));
-    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8+32];"
-        : "=f"(n.c.x), "=f"(n.c.y), "=f"(n.c.z), "=f"(n.c.w), "=r"(n.d.x), "=r"(n.d.y), "=r"(n.d.z), "=r"(n.d.w)
-        : "l"(p));
+    if (SLIM) {
+        n.c = __ldg(&p->c);
+        const int2 d = __ldg(reinterpret_cast<const int2*>(&p->d));
+        n.d = make_int4(d.x, d.y, 0, 0);
+    } else {
+        asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8+32];"
+            : "=f"(n.c.x), "=f"(n.c.y), "=f"(n.c.z), "=f"(n.c.w), "=r"(n.d.x), "=r"(n.d.y), "=r"(n.d.z), "=r"(n.d.w)
+            : "l"(p));
+    }
     return n;
 }
 
@@ -549,7 +560,7 @@ struct WalkStats {
 // pops as selects instead of branches (29.2), a sample queue per lane so that
 // lanes wait less for the warp's slowest ray (2 to 8 samples: 33-35 ms; the
 // lanes drift apart and no longer visit the same nodes).
-template <bool STATS>
+template <bool STATS, bool SLIM = false>
 __device__ __forceinline__ void warp_walk(const SceneView& sc, const TraceRay& r, int skip, BestHit& best, Walk& w,
                                           int* stack, int32_t* status, WalkStats& ws, bool stop_on_hit = false) {
     for (;;) {
@@ -557,7 +568,7 @@ __device__ __forceinline__ void warp_walk(const SceneView& sc, const TraceRay& r
 #pragma unroll
         for (int u = 0; u < WALK_UNROLL; ++u) {
             if ((unsigned)w.node < (unsigned)sc.n_inner) {
-                const BvhNode n = load_node(sc.nodes, w.node);
+                const BvhNode n = load_node<SLIM>(sc.nodes, w.node);
                 if (STATS) ++ws.nodes;
                 ++w.steps;
                 bool h0, h1;
