@@ -66,8 +66,20 @@ k_render_fwd(const float* __restrict__ Ld, const float* __restrict__ Ls0, const 
 constexpr int SUM_THREADS = RENDER_SUM_THREADS;
 __global__ void __launch_bounds__(SUM_THREADS) k_sum_partials(const double* __restrict__ partial, int64_t n,
                                                              double* __restrict__ out) {
+    // a thread's additions are one chain, so its loads go ahead of them in
+    // batches (49,920 partials: 46 us with 128 threads and a load an addition, 39
+    // with batches, 21 with the 1,024 threads of RENDER_SUM_THREADS too)
+    constexpr int AHEAD = 16;
     double s = 0.0;
-    for (int64_t i = threadIdx.x; i < n; i += SUM_THREADS) s += partial[i];
+    int64_t i = threadIdx.x;
+    for (; i + (AHEAD - 1) * SUM_THREADS < n; i += AHEAD * SUM_THREADS) {
+        double v[AHEAD];
+#pragma unroll
+        for (int k = 0; k < AHEAD; ++k) v[k] = partial[i + k * SUM_THREADS];
+#pragma unroll
+        for (int k = 0; k < AHEAD; ++k) s += v[k];
+    }
+    for (; i < n; i += SUM_THREADS) s += partial[i];
     s = warp_sum_down(s);
     __shared__ double ws[SUM_THREADS / 32];
     if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = s;

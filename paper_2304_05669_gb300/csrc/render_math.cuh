@@ -14,7 +14,7 @@
 namespace fipt_render {
 
 constexpr int RENDER_BLOCK = 128;        // points per loss partial (the render kernels' block)
-constexpr int RENDER_SUM_THREADS = 128;  // threads of the final sum over the partials
+constexpr int RENDER_SUM_THREADS = 1024; // threads of the final sum over the partials
 
 struct Grid {
     int K;
