@@ -25,12 +25,14 @@ __all__ = ["Context", "Scene", "bake", "bake_refine", "render_fwd", "render_bwd"
 
 
 def _ptr(t):
-    return ctypes.c_void_p(t.data_ptr()) if t is not None else ctypes.c_void_p(0)
+    return t.data_ptr() if t is not None else None
 
 
 def _stream(stream=None):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    # the current stream's handle without the Stream object around it (10 us on the GB300's host cores)
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _dev(t, dtype, name):
@@ -43,6 +45,8 @@ def _dev(t, dtype, name):
 
 def _need(t, dtype, name, shape):
     """A CUDA tensor of this dtype and exact shape (contiguous; copied if not)."""
+    if isinstance(t, torch.Tensor) and t.is_cuda and t.dtype is dtype and t.shape == shape and t.is_contiguous():
+        return t
     t = _dev(t, dtype, name)
     if tuple(t.shape) != tuple(int(d) for d in shape):
         raise ValueError("%s must have shape %s, got %s" % (name, tuple(shape), tuple(t.shape)))
@@ -71,7 +75,7 @@ def _workspace(nbytes, device):
     """A byte tensor whose data pointer is 256-byte aligned."""
     buf = torch.empty(int(nbytes) + 256, dtype=torch.uint8, device=device)
     off = (-buf.data_ptr()) % 256
-    return buf, buf[off:off + int(nbytes)]
+    return buf, buf[off:off + int(nbytes)] if off else buf
 
 
 class Context:
@@ -438,7 +442,7 @@ def render_fwd(Ld, Ls0, Ls1, sigma_grid, albedo, rough, metal, Lgt=None, mask=No
         Lr = torch.empty((N, 3), dtype=torch.float32, device=Ld.device)
     elif not (Lr.is_cuda and Lr.dtype == torch.float32 and tuple(Lr.shape) == (N, 3) and Lr.is_contiguous()):
         raise ValueError("Lr must be a contiguous CUDA float32 [N, 3] tensor")
-    loss = torch.zeros(1, dtype=torch.float64, device=Ld.device) if Lgt is not None else None
+    loss = torch.empty(1, dtype=torch.float64, device=Ld.device) if Lgt is not None else None
     nbytes = ctypes.c_size_t()
     check(lib().fipt_render_workspace_size(N, ctypes.byref(nbytes)))
     _b, ws = _workspace(nbytes.value, Ld.device)
@@ -478,7 +482,7 @@ def render_fwd_grad(Ld, Ls0, Ls1, sigma_grid, albedo, rough, metal, Lgt, mask=No
     Ld, Ls0, Ls1, albedo, rough, metal, Lgt, mask = _render_inputs(N, K, Ld, Ls0, Ls1, albedo, rough,
                                                                    metal, Lgt, mask)
     Lr = torch.empty((N, 3), dtype=torch.float32, device=Ld.device)
-    loss = torch.zeros(1, dtype=torch.float64, device=Ld.device)
+    loss = torch.empty(1, dtype=torch.float64, device=Ld.device)      # written for every N
     ga = torch.empty((N, 3), dtype=torch.float32, device=Ld.device)
     gr = torch.empty(N, dtype=torch.float32, device=Ld.device)
     gm = torch.empty(N, dtype=torch.float32, device=Ld.device)
@@ -518,22 +522,21 @@ class FactorizedRender(torch.autograd.Function):
             _, loss, ctx.grads = render_fwd_grad(Ld, Ls0, Ls1, sigma_grid, albedo, rough, metal, Lgt, mask)
         else:
             _, loss = render_fwd(Ld, Ls0, Ls1, sigma_grid, albedo, rough, metal, Lgt, mask)
-        ctx.save_for_backward(albedo, rough, metal, Ld, Ls0, Ls1, Lgt,
-                              mask if mask is not None else torch.empty(0, device=Ld.device))
-        ctx.has_mask = mask is not None
+        ctx.save_for_backward(albedo, rough, metal, Ld, Ls0, Ls1, Lgt, mask)
         ctx.sigma_grid = list(sigma_grid)
         return loss[0]
 
     @staticmethod
     def backward(ctx, grad_out):
-        g = grad_out.detach().to(torch.float64).reshape(1).contiguous()
+        g = grad_out.reshape(1)
+        if g.dtype is not torch.float64:
+            g = g.to(torch.float64)
         if ctx.grads is not None:        # computed by the forward pass; handed out once
             grads, ctx.grads = ctx.grads, None
             ga, gr, gm = render_grad_scale(grads, g)
         else:
             albedo, rough, metal, Ld, Ls0, Ls1, Lgt, mask = ctx.saved_tensors
-            ga, gr, gm = render_bwd(Ld, Ls0, Ls1, ctx.sigma_grid, albedo, rough, metal, Lgt,
-                                    mask if ctx.has_mask else None, g)
+            ga, gr, gm = render_bwd(Ld, Ls0, Ls1, ctx.sigma_grid, albedo, rough, metal, Lgt, mask, g)
         return ga, gr, gm, None, None, None, None, None, None
 
 
