@@ -62,6 +62,17 @@ __device__ __forceinline__ long long term(float v, int emin) {
     return (b >> 31) ? -t : t;
 }
 
+// acc + term(v, emin) by one multiply-add: the signed mantissa times
+// 2^(exponent - emin), which is 0 for a zero v (its exponent lies below emin
+// and the shift gives 0 from 32 on).
+__device__ __forceinline__ long long add_term(long long acc, float v, int emin) {
+    const uint32_t b = __float_as_uint(v);
+    const int m = (int)((b & 0x7FFFFFu) | 0x800000u);
+    int p;
+    asm("shl.b32 %0, 1, %1;" : "=r"(p) : "r"((int)((b >> 23) & 0xFFu) - emin));
+    return acc + (long long)((int)b < 0 ? -m : m) * p;
+}
+
 // acc * 2^(emin - 150) as a double (|acc| < 2^53: exact), built from its
 // bits; an exact cancellation gives +0 as FP64 addition does.
 __device__ __forceinline__ double scaled_double(long long acc, int emin) {

@@ -152,84 +152,100 @@ k_vox_compact(const uint32_t* __restrict__ keys, int64_t P, const uint32_t* __re
     if (h) heads[toff[blockIdx.x] + ws[threadIdx.x >> 5] + __popc(m & ((1u << lane) - 1u))] = (uint32_t)j;
 }
 
-#ifndef FIPT_VOX_THREADS
-#define FIPT_VOX_THREADS 64      // small blocks: a long run holds few other runs' slots
-#endif
-#ifndef FIPT_VOX_UNROLL
-#define FIPT_VOX_UNROLL 8        // pixels per group
-#endif
-constexpr int MEAN_THREADS = FIPT_VOX_THREADS;
-constexpr int VU = FIPT_VOX_UNROLL;
+constexpr int MEAN_THREADS = 128;
+constexpr int MEAN_LANES = 8;    // lanes per run
+constexpr int VU = 4;            // pixels a lane takes at a time
 
-// A thread per voxel run: the run's pixels are taken VU at a time, the next
-// group's pixel indices loading while this group's radiance is fetched, and
-// each channel's FP64 sum in pixel order is carried exactly in integers
-// (exact_sum.cuh) while the run's exponent range allows it.  emin and emax
-// are tracked over the three channels together, and the sums are rescaled
-// when a group brings a smaller exponent.  A run that leaves the exact range
-// is summed again with FP64 additions in pixel order.
+// MEAN_LANES lanes per voxel run, which take its pixels MEAN_LANES * VU at a
+// time, the next pixel indices loading while this group's radiance is
+// fetched.  Each channel's FP64 sum in pixel order is carried exactly in
+// integers (exact_sum.cuh), which add up in any order: a lane keeps its own
+// smallest exponent (over the three channels together) and rescales its sums
+// when a group brings a smaller one, and the lanes' sums meet at the run's
+// smallest.  A run that leaves the exact range is summed again with FP64
+// additions in pixel order.  The kernel is bound by its longest runs (4,194,304
+// pixels of the room in 256^3 cells: 210 us with a lane per run, 17 % of the
+// warps active -> 62 us), then by the gathers; lanes 0 to 2 divide a channel
+// each.
 __global__ void __launch_bounds__(MEAN_THREADS)
 k_vox_means(const uint32_t* __restrict__ keys, const uint32_t* __restrict__ pix, const uint32_t* __restrict__ heads,
             const uint32_t* __restrict__ nhead, const float* __restrict__ L, float4* __restrict__ grid) {
+    constexpr unsigned FULL = 0xffffffffu;
+    constexpr int STEP = MEAN_LANES * VU;
     const int64_t nh = *nhead;
-    for (int64_t h = blockIdx.x * (int64_t)MEAN_THREADS + threadIdx.x; h < nh;
-         h += (int64_t)gridDim.x * MEAN_THREADS) {
-        const int64_t j0 = heads[h], j1 = heads[h + 1];
-        const uint32_t k = keys[j0];
+    const int c = threadIdx.x % MEAN_LANES;
+    const int64_t runs = (int64_t)gridDim.x * MEAN_THREADS / MEAN_LANES;
+    // the lanes of a warp go round together (runs past nh are empty)
+    for (int64_t h = (blockIdx.x * (int64_t)MEAN_THREADS + threadIdx.x) / MEAN_LANES;
+         __any_sync(FULL, h < nh); h += runs) {
+        const int64_t j0 = h < nh ? heads[h] : 0, j1 = h < nh ? heads[h + 1] : 0;
+        const int64_t count = j1 - j0;
         long long acc[3] = {0, 0, 0};
         int emin = fipt_exact::EMPTY_EMIN;
         fipt_exact::Range run;
-        bool ok = fipt_exact::spread_limit(j1 - j0) >= 0;
+        bool ok = fipt_exact::spread_limit(count) >= 0;
         uint32_t qn[VU];
 #pragma unroll
-        for (int u = 0; u < VU; ++u) qn[u] = j0 + u < j1 ? pix[j0 + u] : 0u;
-        for (int64_t e = j0; e < j1 && ok; e += VU) {
+        for (int u = 0; u < VU; ++u) {
+            const int64_t e = j0 + c + u * MEAN_LANES;
+            qn[u] = e < j1 ? pix[e] : 0u;
+        }
+        for (int64_t e = j0 + c; e < j1 && ok; e += STEP) {
             float v[VU][3];
 #pragma unroll
             for (int u = 0; u < VU; ++u) {
                 const int64_t q = 3 * (int64_t)qn[u];
-                const bool in = e + u < j1;
+                const bool in = e + u * MEAN_LANES < j1;
                 v[u][0] = in ? L[q] : 0.0f;
                 v[u][1] = in ? L[q + 1] : 0.0f;
                 v[u][2] = in ? L[q + 2] : 0.0f;
             }
 #pragma unroll
-            for (int u = 0; u < VU; ++u) qn[u] = e + VU + u < j1 ? pix[e + VU + u] : 0u;
+            for (int u = 0; u < VU; ++u) {
+                const int64_t x = e + STEP + u * MEAN_LANES;
+                qn[u] = x < j1 ? pix[x] : 0u;
+            }
 #pragma unroll
             for (int u = 0; u < VU; ++u)
 #pragma unroll
-                for (int c = 0; c < 3; ++c) run.note(v[u][c]);
+                for (int k = 0; k < 3; ++k) run.note(v[u][k]);
             const int em = run.emin();
             if (em < emin) {            // from EMPTY_EMIN the sums are still 0
                 const int sh = min(emin - em, 63);
 #pragma unroll
-                for (int c = 0; c < 3; ++c) acc[c] = (long long)((unsigned long long)acc[c] << sh);
+                for (int k = 0; k < 3; ++k) acc[k] = (long long)((unsigned long long)acc[k] << sh);
                 emin = em;
             }
-            ok = !run.special() && run.exact_for(j1 - j0);
+            ok = !run.special() && run.exact_for(count);
             if (ok) {
 #pragma unroll
                 for (int u = 0; u < VU; ++u)
 #pragma unroll
-                    for (int c = 0; c < 3; ++c) acc[c] += fipt_exact::term(v[u][c], emin);
+                    for (int k = 0; k < 3; ++k) acc[k] = fipt_exact::add_term(acc[k], v[u][k], emin);
             }
         }
-        double s0, s1, s2;
-        if (ok) {
-            s0 = fipt_exact::scaled_double(acc[0], emin);
-            s1 = fipt_exact::scaled_double(acc[1], emin);
-            s2 = fipt_exact::scaled_double(acc[2], emin);
-        } else {
-            s0 = s1 = s2 = 0.0;
-            for (int64_t e = j0; e < j1; ++e) {
-                const int64_t q = 3 * (int64_t)pix[e];
-                s0 += (double)L[q];
-                s1 += (double)L[q + 1];
-                s2 += (double)L[q + 2];
-            }
+        // the run's range and sums over its lanes
+#pragma unroll
+        for (int o = 1; o < MEAN_LANES; o <<= 1) {
+            run.lo = min(run.lo, __shfl_xor_sync(FULL, run.lo, o));
+            run.hi = max(run.hi, __shfl_xor_sync(FULL, run.hi, o));
         }
-        const double n = (double)(j1 - j0);
-        grid[k] = make_float4((float)(s0 / n), (float)(s1 / n), (float)(s2 / n), (float)n);
+        const unsigned lanes = ((1u << MEAN_LANES) - 1u) << (threadIdx.x & 31 & ~(MEAN_LANES - 1));
+        ok = (__ballot_sync(FULL, ok) & lanes) == lanes && !run.special() && run.exact_for(count);
+        const int least = run.emin();
+        const int sh = ok ? emin - least : 0;              // 0 to 29 where the lane has a nonzero value
+        double s = 0.0;                                    // lane k: channel k's sum
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            long long a = acc[k] == 0 ? 0 : (long long)((unsigned long long)acc[k] << min(sh, 63));
+#pragma unroll
+            for (int o = 1; o < MEAN_LANES; o <<= 1) a += __shfl_xor_sync(FULL, a, o);
+            if (c == k && ok) s = fipt_exact::scaled_double(a, least);
+        }
+        if (!ok && c < 3)
+            for (int64_t e = j0; e < j1; ++e) s += (double)L[3 * (int64_t)pix[e] + c];
+        const float m = c < 3 ? (float)(s / (double)(count > 0 ? count : 1)) : (float)count;
+        if (h < nh && c < 4) reinterpret_cast<float*>(grid + keys[j0])[c] = m;
     }
 }
 
