@@ -59,15 +59,16 @@ __global__ void k_debug_divide(DivN d, const uint32_t* __restrict__ i, int64_t c
 
 // IDX: uint32_t when T * n < 2^32 (the sample index splits by the
 // multiply-high division above), int64_t otherwise.  Bound by the
-// instructions of a sample's ten Philox rounds and its square root, then by
-// the 12 bytes written, so a thread takes PTS_PER consecutive samples: the
-// index is divided and the triangle loaded once, and the block's points,
-// contiguous in x, leave shared memory in one bulk copy (x 16-byte aligned)
-// instead of by loads and stores.  204,546,400 points (100 on each triangle
-// of the floor): 1,062 -> 828 us (363 us at the copy rate), one point
-// per thread and float4 stores before.
-constexpr int PTS_THREADS = 256;
-constexpr int PTS_PER = 4;
+// instructions of a sample's ten Philox rounds and its square root and by the
+// latency of the triangle's records, then by the 12 bytes written; so a thread
+// takes PTS_PER consecutive samples: the index is divided and the triangle
+// loaded once, and the block's points, contiguous in x, leave shared memory in
+// one bulk copy (x 16-byte aligned) instead of by loads and stores.
+// 204,546,400 points (100 on each triangle of the floor; 363 us at the copy
+// rate): 1,062 us with a point per thread and float4 stores, 821 / 726 with 4 per
+// thread in blocks of 256 / 128, 690 / 670 with 8.
+constexpr int PTS_THREADS = 128;
+constexpr int PTS_PER = 8;
 constexpr int PTS_BLOCK = PTS_THREADS * PTS_PER;
 
 template <class IDX>
@@ -194,6 +195,84 @@ k_emit_classify(const float* __restrict__ alpha, int64_t T, int n, double thr,
         for (int j = 0; j < n; ++j) s += (double)row[j];
     }
     const double m = s / (double)n;
+    if (mean) mean[t] = m;
+    flag[t] = m > thr ? 1 : 0;
+}
+
+// Rows of a multiple of 4 samples, at most 4 * ROW_V * ROW_LANES of them,
+// 16-byte aligned: ROW_LANES lanes hold a row in registers, so every sample is
+// loaded once, by independent 16-byte loads, and nothing waits on shared
+// memory; the exponent range and the integer sum (exact_sum.cuh) are then taken
+// over the lanes.  Adding a term is one 32 x 32 + 64-bit multiply-add by a
+// power of two.  A warp takes 32 rows, so that the FP64 division of each is a
+// lane's.  100 samples on 2,045,464 triangles: 309 us staged (ALU-bound on
+// 64-bit shifts, 17 % of the warps) -> 186 us, 121 at the copy rate.
+constexpr int ROW_THREADS = 128;
+constexpr int ROW_LANES = 4;
+constexpr int ROW_V = 8;
+constexpr int ROW_MAX = 4 * ROW_V * ROW_LANES;
+
+__global__ void __launch_bounds__(ROW_THREADS)
+k_emit_classify_rows(const float4* __restrict__ alpha, int64_t T, int n, double thr, double* __restrict__ mean,
+                     uint8_t* __restrict__ flag) {
+    constexpr unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, c = lane % ROW_LANES;
+    const int64_t t0 = (blockIdx.x * (int64_t)ROW_THREADS + threadIdx.x) & ~int64_t(31);
+    if (t0 >= T) return;                                   // whole warp
+    const int n4 = n >> 2;
+    double mine = 0.0;                                     // the sum of row t0 + lane
+#pragma unroll 1
+    for (int r = 0; r < ROW_LANES; ++r) {
+        const int64_t t = t0 + r * (32 / ROW_LANES) + lane / ROW_LANES;
+        const float4* row = alpha + t * n4;
+        float4 v[ROW_V];
+#pragma unroll
+        for (int k = 0; k < ROW_V; ++k) {
+            const int i = c + ROW_LANES * k;
+            v[k] = t < T && i < n4 ? __ldg(row + i) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        }
+        fipt_exact::Range rg;
+#pragma unroll
+        for (int k = 0; k < ROW_V; ++k) {
+            rg.note(v[k].x);
+            rg.note(v[k].y);
+            rg.note(v[k].z);
+            rg.note(v[k].w);
+        }
+#pragma unroll
+        for (int o = 1; o < ROW_LANES; o <<= 1) {
+            rg.lo = min(rg.lo, __shfl_xor_sync(FULL, rg.lo, o));
+            rg.hi = max(rg.hi, __shfl_xor_sync(FULL, rg.hi, o));
+        }
+        double s;
+        if (!rg.special() && rg.exact_for(n)) {
+            const int emin = rg.emin();
+            long long acc = 0;
+#pragma unroll
+            for (int k = 0; k < ROW_V; ++k) {
+                acc = fipt_exact::add_term(acc, v[k].x, emin);
+                acc = fipt_exact::add_term(acc, v[k].y, emin);
+                acc = fipt_exact::add_term(acc, v[k].z, emin);
+                acc = fipt_exact::add_term(acc, v[k].w, emin);
+            }
+            // the lanes of a row take this branch together
+            const unsigned group = ((1u << ROW_LANES) - 1u) << (lane & ~(ROW_LANES - 1));
+#pragma unroll
+            for (int o = 1; o < ROW_LANES; o <<= 1) acc += __shfl_xor_sync(group, acc, o);
+            s = fipt_exact::scaled_double(acc, emin);
+        } else {
+            s = 0.0;
+            const float* x = reinterpret_cast<const float*>(row);
+            if (c == 0)
+                for (int j = 0; j < n; ++j) s += (double)x[j];
+        }
+        __syncwarp();
+        const double got = __shfl_sync(FULL, s, lane % (32 / ROW_LANES) * ROW_LANES);
+        if (lane / (32 / ROW_LANES) == r) mine = got;
+    }
+    const int64_t t = t0 + lane;
+    if (t >= T) return;
+    const double m = mine / (double)n;
     if (mean) mean[t] = m;
     flag[t] = m > thr ? 1 : 0;
 }
@@ -521,7 +600,10 @@ extern "C" fipt_status fipt_emitter_classify(const float* alpha, int64_t T, int3
     FIPT_REQUIRE(!mean_alpha || fipt_aligned(mean_alpha, 8), "mean_alpha misaligned");
     const unsigned nb = blocks(T, CLS_THREADS);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (n_per_tri <= CLS_STAGE_N)
+    if (n_per_tri % 4 == 0 && n_per_tri <= ROW_MAX && fipt_aligned(alpha, 16))
+        FIPT_LAUNCH(k_emit_classify_rows, blocks(T, ROW_THREADS), ROW_THREADS, 0, st,
+                    reinterpret_cast<const float4*>(alpha), T, n_per_tri, (double)threshold, mean_alpha, is_emitter);
+    else if (n_per_tri <= CLS_STAGE_N)
         FIPT_LAUNCH(k_emit_classify<true>, nb, CLS_THREADS, 0, st, alpha, T, n_per_tri, (double)threshold,
                     mean_alpha, is_emitter);
     else
