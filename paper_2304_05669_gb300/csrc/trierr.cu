@@ -18,13 +18,22 @@ __global__ void k_tri_keys(const int32_t* __restrict__ tri, int64_t stride, int6
     vals[p] = (uint32_t)p;
 }
 
+// A float as a double by integer operations (FP64 conversions run at the rate
+// of FP64 additions); subnormals, infinities and NaNs are converted.
+__device__ __forceinline__ double widen(float f) {
+    const uint32_t b = __float_as_uint(f);
+    if (((b >> 23) & 0xffu) - 1u < 254u)
+        return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+    return (b << 1) == 0u ? __hiloint2double((int)b, 0) : (double)f;
+}
+
 // One warp per TILE sorted pixels.  The kernel is bound by FP64 (1/64 of the
-// float32 rate), so its lanes are pixels, all of them busy: 18 FP64
+// float32 rate), so its lanes are pixels, all of them busy: 12 FP64
 // instructions per row of 32 pixels, however long the segments are.  (A warp
 // per triangle spent five additions of its butterfly on each of the floor's
 // 2,045,464 triangles, most of them unseen, and a lane of it 3,000 dependent
 // gathers on a triangle that 100,000 pixels see: 2,636 us for 4,194,304
-// pixels against 153 us here.)
+// pixels against 153 us here, 107 since the floats widen by integer operations.)
 //
 // A segment inside the tile is written at its last pixel.  head_sum / head_end
 // [w]: the part in tile w of a segment that began before it, and the position
@@ -60,7 +69,7 @@ k_tile_sums(const uint32_t* __restrict__ keys, const uint32_t* __restrict__ pix,
             const int64_t p = pix[j];
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                const double d = (double)Lr[3 * p + c] - (double)Lgt[3 * p + c];
+                const double d = widen(Lr[3 * p + c]) - widen(Lgt[3 * p + c]);
                 v = fma(d, d, v);
             }
         }
