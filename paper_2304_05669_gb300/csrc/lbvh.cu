@@ -38,30 +38,6 @@ k_sort_hist(const K* __restrict__ keys, int64_t n, const uint32_t* __restrict__ 
     hist[(int64_t)threadIdx.x * gridDim.x + blockIdx.x] = cnt[threadIdx.x];
 }
 
-// Exclusive scan of m counters in one block (digit-major histogram).
-__global__ void __launch_bounds__(SCAN_THREADS) k_scan_single(uint32_t* __restrict__ a, int64_t m) {
-    __shared__ uint32_t part[SCAN_THREADS];
-    const int64_t per = (m + SCAN_THREADS - 1) / SCAN_THREADS;
-    const int64_t beg = threadIdx.x * per;
-    const int64_t end = beg + per < m ? beg + per : m;
-    uint32_t s = 0;
-    for (int64_t i = beg; i < end; ++i) s += a[i];
-    part[threadIdx.x] = s;
-    __syncthreads();
-    for (int off = 1; off < SCAN_THREADS; off <<= 1) {
-        uint32_t v = threadIdx.x >= off ? part[threadIdx.x - off] : 0u;
-        __syncthreads();
-        part[threadIdx.x] += v;
-        __syncthreads();
-    }
-    uint32_t run = part[threadIdx.x] - s;
-    for (int64_t i = beg; i < end; ++i) {
-        const uint32_t v = a[i];
-        a[i] = run;
-        run += v;
-    }
-}
-
 // Multi-block exclusive scan for large histograms: k_scan_reduce sums
 // chunks of SCAN_CHUNK counters, k_scan_single scans those sums, and
 // k_scan_apply scans each chunk from its scanned sum.  Thread i of a block
@@ -71,6 +47,57 @@ constexpr int SCAN_CHUNK = 4 * SCAN_THREADS;
 __device__ __forceinline__ uint4 load4(const uint32_t* a, int64_t i, int64_t m) {
     if (i + 3 < m) return *reinterpret_cast<const uint4*>(a + i);
     return make_uint4(i < m ? a[i] : 0u, i + 1 < m ? a[i + 1] : 0u, i + 2 < m ? a[i + 2] : 0u, 0u);
+}
+
+// The block's exclusive scan of its threads' t, plus base; total receives the
+// sum.  wsum: 33 words.
+__device__ __forceinline__ uint32_t scan_threads(uint32_t t, uint32_t base, uint32_t* wsum, uint32_t& total) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t incl = t;
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    if (lane == 31) wsum[warp] = incl;
+    __syncthreads();
+    if (warp == 0) {
+        uint32_t u = wsum[lane];
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, u, o);
+            if (lane >= o) u += y;
+        }
+        wsum[lane] = u;
+    }
+    __syncthreads();
+    total = wsum[SCAN_THREADS / 32 - 1];
+    return base + (warp > 0 ? wsum[warp - 1] : 0u) + incl - t;
+}
+
+__device__ __forceinline__ void store4(uint32_t* a, int64_t i, int64_t m, uint32_t run, uint4 v) {
+    const uint32_t e0 = run, e1 = e0 + v.x, e2 = e1 + v.y, e3 = e2 + v.z;
+    if (i + 3 < m) {
+        *reinterpret_cast<uint4*>(a + i) = make_uint4(e0, e1, e2, e3);
+    } else {
+        if (i < m) a[i] = e0;
+        if (i + 1 < m) a[i + 1] = e1;
+        if (i + 2 < m) a[i + 2] = e2;
+    }
+}
+
+// Exclusive scan of m counters by one block, chunk after chunk (16,384
+// counters: 24 us with each thread summing its own stretch -> 5 us).
+__global__ void __launch_bounds__(SCAN_THREADS) k_scan_single(uint32_t* __restrict__ a, int64_t m) {
+    __shared__ uint32_t wsum[SCAN_THREADS / 32];
+    uint32_t carry = 0;
+    for (int64_t base = 0; base < m; base += SCAN_CHUNK) {
+        const int64_t i = base + 4 * threadIdx.x;
+        const uint4 v = load4(a, i, m);
+        uint32_t total;
+        const uint32_t run = scan_threads(v.x + v.y + v.z + v.w, carry, wsum, total);
+        store4(a, i, m, run, v);
+        carry += total;
+        __syncthreads();                                    // wsum is rewritten by the next chunk
+    }
 }
 
 __global__ void __launch_bounds__(SCAN_THREADS)
@@ -92,35 +119,10 @@ k_scan_reduce(const uint32_t* __restrict__ a, int64_t m, uint32_t* __restrict__ 
 __global__ void __launch_bounds__(SCAN_THREADS)
 k_scan_apply(uint32_t* __restrict__ a, int64_t m, const uint32_t* __restrict__ bsum) {
     __shared__ uint32_t wsum[SCAN_THREADS / 32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t i = (int64_t)blockIdx.x * SCAN_CHUNK + 4 * threadIdx.x;
     const uint4 v = load4(a, i, m);
-    const uint32_t t = v.x + v.y + v.z + v.w;
-    uint32_t incl = t;
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += y;
-    }
-    if (lane == 31) wsum[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-        uint32_t u = wsum[lane];
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, u, o);
-            if (lane >= o) u += y;
-        }
-        wsum[lane] = u;
-    }
-    __syncthreads();
-    uint32_t run = bsum[blockIdx.x] + (warp > 0 ? wsum[warp - 1] : 0u) + incl - t;
-    const uint32_t e0 = run, e1 = e0 + v.x, e2 = e1 + v.y, e3 = e2 + v.z;
-    if (i + 3 < m) {
-        *reinterpret_cast<uint4*>(a + i) = make_uint4(e0, e1, e2, e3);
-    } else {
-        if (i < m) a[i] = e0;
-        if (i + 1 < m) a[i + 1] = e1;
-        if (i + 2 < m) a[i + 2] = e2;
-    }
+    uint32_t total;
+    store4(a, i, m, scan_threads(v.x + v.y + v.z + v.w, bsum[blockIdx.x], wsum, total), v);
 }
 
 // The stable order of a block's keys by one digit.  A warp holds 32 * ITEMS
