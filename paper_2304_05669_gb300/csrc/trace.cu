@@ -12,8 +12,9 @@
 namespace {
 
 constexpr int TRACE_THREADS = 128;
+constexpr int TRACE_MINB = 12;       // resident blocks per SM (40 registers; 10 at 48: first hits 0.894 against 0.858 ms)
 
-__global__ void __launch_bounds__(TRACE_THREADS)
+__global__ void __launch_bounds__(TRACE_THREADS, TRACE_MINB)
 k_trace(SceneView sc, const float* __restrict__ orig, const float* __restrict__ dir, int64_t n,
         const int32_t* __restrict__ skip, int32_t* __restrict__ hit_tri, float* __restrict__ hit_t,
         int32_t* __restrict__ hit_front, int32_t* status) {
@@ -33,7 +34,7 @@ k_trace(SceneView sc, const float* __restrict__ orig, const float* __restrict__ 
 // whose rays walk the tree more alike than those of 32 pixels of a row (24
 // views of 640 x 416 in the room: 820 -> 776 us).  Lanes past the image's
 // edges have no ray.
-__global__ void __launch_bounds__(TRACE_THREADS)
+__global__ void __launch_bounds__(TRACE_THREADS, TRACE_MINB)
 k_camera(SceneView sc, const float* __restrict__ cams, int W, int H, int log_tw, int tiles_x, int tiles_y, int64_t tiles,
          fipt_query* __restrict__ out, int32_t* __restrict__ valid, int32_t* status) {
     const int64_t tile = (blockIdx.x * (int64_t)TRACE_THREADS + threadIdx.x) >> 5;
