@@ -214,14 +214,13 @@ constexpr uint32_t F_DEPTH = 0xffffu;
 constexpr uint32_t F_PATH = 1u << 16, F_SHADOW = 1u << 17, F_AT_X = 1u << 18, F_LIVE = 1u << 19;
 
 struct RfState {
-    float4* org;        // [P] origin of the slot's rays (xyz), the triangle they skip (int bits)
+    // records that are used together lie side by side, a slot's pair in one 32-byte sector
+    float4* os;         // [2P] origin of the slot's rays (xyz), the triangle they skip (int bits); shadow-ray weights
+                        // (rgb), target emitter leaf (int bits)
     float4* dir;        // [2P] ray 2j: path segment, 2j+1: shadow ray; direction (xyz), t_max
     int4* hit;          // [2P] t (float bits), leaf (-1: none), original triangle id, front face
-    float4* bp;         // [P] path throughput (rgb), pdf of the last BRDF sample
-    float4* lw;         // [P] path radiance (rgb), W0
-    float4* c0;         // [P] sample value for L_d / L_s0 (rgb), W1
-    float4* c1;         // [P] sample value for L_s1 (rgb), flags (int bits)
-    float4* sw;         // [P] shadow-ray weights (rgb), target emitter leaf (int bits)
+    float4* lb;         // [2P] path radiance (rgb), W0; path throughput (rgb), pdf of the last BRDF sample
+    float4* cc;         // [2P] sample value for L_d / L_s0 (rgb), W1; for L_s1 (rgb), flags (int bits)
     uint32_t* act[2];   // slots with queued rays, by wave parity
     uint32_t* tq[2];    // queued ray ids, by wave parity
     uint32_t* cnt;      // wave w: [4w] rays queued, [4w+1] rays taken, [4w+2] slots active
@@ -275,6 +274,25 @@ __device__ __forceinline__ void slot_decode(uint32_t j, const RefineArgs& R, uin
         lobe = 1 + r / R.A.spp_s;
         s = r - (lobe - 1) * R.A.spp_s;
     }
+}
+
+// Two neighbouring records in one 32-byte access (p 32-byte aligned: the
+// arrays start 256-byte aligned and pairs at even records).
+__device__ __forceinline__ void load_pair(const float4* p, float4& a, float4& b) {
+    asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
+                 : "l"(p)
+                 : "memory");
+}
+
+__device__ __forceinline__ void store_pair(float4* p, float4 a, float4 b) {
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(a.x), "f"(a.y), "f"(a.z),
+                 "f"(a.w), "f"(b.x), "f"(b.y), "f"(b.z), "f"(b.w)
+                 : "memory");
+}
+
+__device__ __forceinline__ int4 as_int4(float4 v) {
+    return make_int4(__float_as_int(v.x), __float_as_int(v.y), __float_as_int(v.z), __float_as_int(v.w));
 }
 
 // Appends v to list for every lane with pred (one atomic per warp); all 32
@@ -341,7 +359,7 @@ k_rf_gen(SceneView sc, RfChunk C, RefineArgs R, RfState st) {
                 }
                 const uint32_t pid = A.point_base + (uint32_t)pq;
                 const float ox = q0.x + eps * n.x, oy = q0.y + eps * n.y, oz = q1.x + eps * n.z;
-                st.org[j] = make_float4(ox, oy, oz, q4.y);         // q4.y: the query's triangle
+                st.os[2 * j] = make_float4(ox, oy, oz, q4.y);         // q4.y: the query's triangle
                 if (mis) {                                          // emitter sample at x
                     float3 y;
                     const int e = emitter_sample(sc, n_emit, A_emit,
@@ -376,7 +394,7 @@ k_rf_gen(SceneView sc, RfChunk C, RefineArgs R, RfState st) {
                     if (g0 > 0.0f || g1 > 0.0f) {
                         const float pl = dist * dist / (A_emit_f * ce);
                         const float wgt = pl * pl / (pl * pl + pb * pb);
-                        st.sw[j] = make_float4(wgt * g0 / pl, wgt * g1 / pl, 0.0f, __int_as_float(e));
+                        st.os[2 * j + 1] = make_float4(wgt * g0 / pl, wgt * g1 / pl, 0.0f, __int_as_float(e));
                         st.dir[2 * j + 1] = make_float4(ex, ey, ez, 1.001f * dist + eps);
                         flags |= F_SHADOW | F_AT_X;
                         qshadow = true;
@@ -417,16 +435,15 @@ k_rf_gen(SceneView sc, RfChunk C, RefineArgs R, RfState st) {
                 }
                 if (ok) {
                     st.dir[2 * j] = make_float4(wi.x, wi.y, wi.z, FINF);
-                    st.bp[j] = make_float4(1.0f, 1.0f, 1.0f, pb);
-                    st.lw[j] = make_float4(0.0f, 0.0f, 0.0f, W0);
+                    st.lb[2 * j + 1] = make_float4(1.0f, 1.0f, 1.0f, pb);
+                    st.lb[2 * j] = make_float4(0.0f, 0.0f, 0.0f, W0);
                     C0.w = W1;
                     flags |= F_PATH | F_LIVE | 1u;
                     qpath = true;
                 }
             }
             C1.w = __uint_as_float(flags);
-            st.c0[j] = C0;
-            st.c1[j] = C1;
+            store_pair(st.cc + 2 * j, C0, C1);
         }
         warp_append(st.act[0], st.cnt + 2, qpath || qshadow, (uint32_t)j);
         warp_append(st.tq[0], st.cnt + 0, qpath, (uint32_t)(2 * j));
@@ -496,7 +513,7 @@ k_rf_trace(SceneView sc, RfState st, int w, int32_t* status, unsigned long long*
                 const uint32_t i = b + __popc(m_need & ((1u << lane) - 1u));
                 if (i < n) {
                     rid = (int)__ldg(queue + i);
-                    const float4 o = __ldg(st.org + (rid >> 1)), d = __ldg(st.dir + rid);
+                    const float4 o = __ldg(st.os + (rid & ~1)), d = __ldg(st.dir + rid);
                     r = make_ray(o.x, o.y, o.z, d.x, d.y, d.z);
                     skip = __float_as_int(o.w);
                     best.t = d.w;
@@ -505,7 +522,7 @@ k_rf_trace(SceneView sc, RfState st, int w, int32_t* status, unsigned long long*
                     if (STATS) ++n_rays;
                     shadow = (rid & 1) != 0;
                     if (shadow) {                  // settle the target first
-                        const int tgt = __float_as_int(__ldg(&st.sw[rid >> 1].w));
+                        const int tgt = __float_as_int(__ldg(&st.os[rid | 1].w));
                         const float4 p0 = __ldg(sc.tris + 3 * tgt);
                         const int orig = __float_as_int(p0.w);
                         float t;
@@ -568,12 +585,15 @@ k_rf_shade(SceneView sc, RfChunk C, RefineArgs R, RfState st, int w) {
             int lobe, s;
             slot_decode(j, R, (uint32_t)C.n_pts, pc, lobe, s);
             const uint32_t pid = A.point_base + (uint32_t)C.point(pc);
-            float4 C0 = st.c0[j], C1 = st.c1[j], LW = st.lw[j];
+            float4 C0, C1, LW, BP, O, SW, h0, h1;
+            load_pair(st.cc + 2 * j, C0, C1);
             // the slot's other records, loaded together whether or not a ray
             // of their kind was queued (they are unused then)
-            const float4 SW = st.sw[j], D = st.dir[2 * j], O = st.org[j];
-            const int4 hs = st.hit[2 * j + 1], h = st.hit[2 * j];
-            const float4 BP = st.bp[j];
+            load_pair(st.lb + 2 * j, LW, BP);
+            load_pair(st.os + 2 * j, O, SW);
+            load_pair(reinterpret_cast<const float4*>(st.hit) + 2 * j, h0, h1);
+            const float4 D = st.dir[2 * j];
+            const int4 h = as_int4(h0), hs = as_int4(h1);
             const uint32_t f_in = __float_as_uint(C1.w);
             uint32_t depth = f_in & F_DEPTH;
             uint32_t flags = f_in & F_LIVE;
@@ -624,7 +644,7 @@ k_rf_shade(SceneView sc, RfChunk C, RefineArgs R, RfState st, int w) {
                         float3 nv = tri_normal(p0, p1, p2);
                         if (nv.x * dx + nv.y * dy + nv.z * dz > 0.0f) nv = make_float3(-nv.x, -nv.y, -nv.z);
                         const float xox = hx + eps * nv.x, xoy = hy + eps * nv.y, xoz = hz + eps * nv.z;
-                        st.org[j] = make_float4(xox, xoy, xoz, __int_as_float(h.z));
+                        st.os[2 * j] = make_float4(xox, xoy, xoz, __int_as_float(h.z));
                         const float3 wv = make_float3(-dx, -dy, -dz);
                         const float mu_v = nv.x * wv.x + nv.y * wv.y + nv.z * wv.z;
                         const Mat M = vertex_mat(m0, m1, mu_v);
@@ -643,7 +663,7 @@ k_rf_shade(SceneView sc, RfChunk C, RefineArgs R, RfState st, int w) {
                                 if (f[0] > 0.0f || f[1] > 0.0f || f[2] > 0.0f) {
                                     const float pl = dist * dist / (A_emit_f * ce);
                                     const float wgt = pl * pl / (pl * pl + pb * pb);
-                                    st.sw[j] = make_float4(BP.x * wgt * f[0] / pl, BP.y * wgt * f[1] / pl,
+                                    st.os[2 * j + 1] = make_float4(BP.x * wgt * f[0] / pl, BP.y * wgt * f[1] / pl,
                                                            BP.z * wgt * f[2] / pl, __int_as_float(e));
                                     st.dir[2 * j + 1] = make_float4(ex, ey, ez, 1.001f * dist + eps);
                                     flags |= F_SHADOW;
@@ -674,7 +694,7 @@ k_rf_shade(SceneView sc, RfChunk C, RefineArgs R, RfState st, int w) {
                         float f[3], pdf;
                         vertex_brdf(M, nv, wv, wi, mu_v, f, pdf, glossy, hh, sin2h);
                         if (pdf > 0.0f) {
-                            st.bp[j] = make_float4(BP.x * (f[0] / pdf), BP.y * (f[1] / pdf), BP.z * (f[2] / pdf), pdf);
+                            st.lb[2 * j + 1] = make_float4(BP.x * (f[0] / pdf), BP.y * (f[1] / pdf), BP.z * (f[2] / pdf), pdf);
                             st.dir[2 * j] = make_float4(wi.x, wi.y, wi.z, FINF);
                             ++depth;
                             flags |= F_PATH;
@@ -690,9 +710,8 @@ k_rf_shade(SceneView sc, RfChunk C, RefineArgs R, RfState st, int w) {
                 flags &= ~F_LIVE;
             }
             C1.w = __uint_as_float(flags | depth);
-            st.c0[j] = C0;
-            st.c1[j] = C1;
-            st.lw[j] = LW;
+            store_pair(st.cc + 2 * j, C0, C1);
+            st.lb[2 * j] = LW;
         }
         warp_append(nact, ncnt + 2, qpath || qshadow, j);
         warp_append(ntq, ncnt + 0, qpath, 2 * j);
@@ -720,7 +739,8 @@ k_rf_reduce(RfChunk C, RefineArgs R, RfState st, float* __restrict__ Ld, float* 
     float* ps = PER_SAMPLE ? per_sample + (size_t)(p * L + lobe) * R.smax * 6 : nullptr;
     for (int s = 0; s < S; ++s) {
         const uint32_t j = slot_of((uint32_t)pc, (uint32_t)(r0 + s), R, (uint32_t)C.n_pts);
-        const float4 x = st.c0[j], y = st.c1[j];
+        float4 x, y;
+        load_pair(st.cc + 2 * j, x, y);
         a0 += x.x; a1 += x.y; a2 += x.z;
         a3 += y.x; a4 += y.y; a5 += y.z;
         if (PER_SAMPLE) {
@@ -756,14 +776,11 @@ struct RfLayout {
 RfLayout carve_refine(void* base, int64_t N, int64_t P, int waves) {
     Carver c{static_cast<char*>(base), 0};
     RfLayout L;
-    L.st.org = c.take<float4>(P);
+    L.st.os = c.take<float4>(2 * P);
     L.st.dir = c.take<float4>(2 * P);
     L.st.hit = c.take<int4>(2 * P);
-    L.st.bp = c.take<float4>(P);
-    L.st.lw = c.take<float4>(P);
-    L.st.c0 = c.take<float4>(P);
-    L.st.c1 = c.take<float4>(P);
-    L.st.sw = c.take<float4>(P);
+    L.st.lb = c.take<float4>(2 * P);
+    L.st.cc = c.take<float4>(2 * P);
     L.st.act[0] = c.take<uint32_t>(P);
     L.st.act[1] = c.take<uint32_t>(P);
     L.st.tq[0] = c.take<uint32_t>(2 * P);
