@@ -66,9 +66,10 @@ __global__ void k_debug_divide(DivN d, const uint32_t* __restrict__ i, int64_t c
 // one bulk copy (x 16-byte aligned) instead of by loads and stores.
 // 204,546,400 points (100 on each triangle of the floor; 363 us at the copy
 // rate): 1,062 us with a point per thread and float4 stores, 821 / 726 with 4 per
-// thread in blocks of 256 / 128, 690 / 670 with 8.
+// thread in blocks of 256 / 128, 690 / 670 with 8, 640 with
+// 16 in blocks of 128.
 constexpr int PTS_THREADS = 128;
-constexpr int PTS_PER = 8;
+constexpr int PTS_PER = 16;
 constexpr int PTS_BLOCK = PTS_THREADS * PTS_PER;
 
 template <class IDX>
@@ -89,29 +90,32 @@ k_emit_points(const float4* __restrict__ tris, const int32_t* __restrict__ inv, 
         int j = (int)((IDX)i - t * (IDX)n);
         int leaf = inv[t];
         float4 p0 = __ldg(tris + 3 * leaf), p1 = __ldg(tris + 3 * leaf + 1), p2 = __ldg(tris + 3 * leaf + 2);
-        float v[3 * PTS_PER];
-#pragma unroll
-        for (int q = 0; q < PTS_PER; ++q) {
-            if (q > 0 && ++j == n) {                       // the next triangle
-                j = 0;
-                if ((int64_t)++t < T) {
-                    leaf = inv[t];
-                    p0 = __ldg(tris + 3 * leaf);
-                    p1 = __ldg(tris + 3 * leaf + 1);
-                    p2 = __ldg(tris + 3 * leaf + 2);
-                }
-            }
-            const uint4 w = philox4x32_10(make_uint4((uint32_t)t, (uint32_t)j, EMIT_LANE, rid), key);
-            const float u1 = u24f(w.x), u2 = u24f(w.y);
-            const float r1 = sqrtf(u1);
-            const float b0 = 1.0f - r1, b1 = r1 * (1.0f - u2), b2 = r1 * u2;
-            v[3 * q + 0] = b0 * p0.x + b1 * p1.x + b2 * p2.x;
-            v[3 * q + 1] = b0 * p0.y + b1 * p1.y + b2 * p2.y;
-            v[3 * q + 2] = b0 * p0.z + b1 * p1.z + b2 * p2.z;
-        }
         float4* dst = reinterpret_cast<float4*>(sb + 3 * PTS_PER * threadIdx.x);
+#pragma unroll 1
+        for (int q4 = 0; q4 < PTS_PER; q4 += 4) {
+            float v[12];
 #pragma unroll
-        for (int q = 0; q < 3 * PTS_PER / 4; ++q) dst[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+            for (int q = 0; q < 4; ++q) {
+                if (q4 + q > 0 && ++j == n) {              // the next triangle
+                    j = 0;
+                    if ((int64_t)++t < T) {
+                        leaf = inv[t];
+                        p0 = __ldg(tris + 3 * leaf);
+                        p1 = __ldg(tris + 3 * leaf + 1);
+                        p2 = __ldg(tris + 3 * leaf + 2);
+                    }
+                }
+                const uint4 w = philox4x32_10(make_uint4((uint32_t)t, (uint32_t)j, EMIT_LANE, rid), key);
+                const float u1 = u24f(w.x), u2 = u24f(w.y);
+                const float r1 = sqrtf(u1);
+                const float b0 = 1.0f - r1, b1 = r1 * (1.0f - u2), b2 = r1 * u2;
+                v[3 * q + 0] = b0 * p0.x + b1 * p1.x + b2 * p2.x;
+                v[3 * q + 1] = b0 * p0.y + b1 * p1.y + b2 * p2.y;
+                v[3 * q + 2] = b0 * p0.z + b1 * p1.z + b2 * p2.z;
+            }
+#pragma unroll
+            for (int q = 0; q < 3; ++q) dst[3 * (q4 >> 2) + q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+        }
     }
     const int64_t here = total - base < PTS_BLOCK ? total - base : PTS_BLOCK;
     if (here == PTS_BLOCK && (reinterpret_cast<uintptr_t>(x) & 15) == 0) {     // the same for the whole block
