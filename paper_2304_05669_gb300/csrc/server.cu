@@ -570,13 +570,19 @@ void fipt_server::stage_chunks() {
     if (order.size() > 1)
         std::stable_sort(order.begin() + 1, order.end(),
                          [&](uint64_t a, uint64_t b) { return remaining(a) < remaining(b); });
+    int64_t pairs_waiting = 0;
+    for (uint64_t t : order) pairs_waiting += (reqs[t]->r.n - reqs[t]->next) * (1 + reqs[t]->r.params.K);
     const int first = n_staged;
     auto take = [&](uint64_t t, int64_t share) {
         Req* q = reqs[t];
         const fipt_bake_params& P = q->r.params;
         const int64_t rpp = rays_per_point(P);
-        const int log_g = bake_split(q->r.n * (1 + P.K), scenes[q->r.target]->T,
-                                     std::min(P.spp_diffuse, P.spp_specular));
+        // the request's own split, but no finer than two lanes a pair where the work waiting would not want it:
+        // with other requests to fill the chip, a small one gains nothing from spreading
+        const int least = std::min(P.spp_diffuse, P.spp_specular);
+        const int64_t T = scenes[q->r.target]->T;
+        const int log_g = std::min(bake_split(q->r.n * (1 + P.K), T, least),
+                                   std::max(bake_split(pairs_waiting, T, least), std::min(least, 2) - 1));
         int64_t got = 0;
         while (q->next < q->r.n && n_staged < kQueue) {
             const int64_t c = std::min<int64_t>(chunk_points, q->r.n - q->next);
