@@ -355,8 +355,8 @@ fipt_status fipt_scene_set_materials(fipt_scene* scene, const float* albedo, con
  * workspace: device, 256-byte aligned, at least the bytes
  * fipt_bake_refine_workspace_size gives for the same N, params and
  * max_depth (the path state of up to 16,777,216 samples at a time, 184
- * bytes each, about 3.1 GB; larger calls run in chunks of whole points);
- * owned by the caller, in use until the stream reaches the end of the call.
+ * bytes each, about 3.1 GB, larger calls running in chunks of whole points,
+ * and 4 bytes a point for their order); owned by the caller, in use until the stream reaches the end of the call.
  * spp_diffuse + K * spp_specular above 16,777,216 is FIPT_ERR_INVALID_ARG;
  * a workspace below the size is FIPT_ERR_WORKSPACE.  max_depth > 15 makes
  * the call wait for the stream every 16 path depths to stop once every
@@ -468,7 +468,8 @@ fipt_status fipt_tri_error(const int32_t* tri, int64_t tri_stride, const float* 
  * warps stay resident on every SM and take warp items as the scheduler
  * publishes them, without a launch per request:
  *  - the bake loop (all block slots of 64 threads but two per SM): warp
- *    items of 32 points of one chunk and one lobe, one atomic add each.
+ *    items of one chunk and one lobe, of 32 points or, where lanes share
+ *    points, as few as one, one atomic add each.
  *    The scheduler keeps bake items published ahead of the loop and not
  *    yet taken -- two per resident warp, and at least max_batch_rays rays
  *    -- in chunks of up to chunk_points points: the oldest request first,

@@ -24,9 +24,8 @@
 //                at x (a shadow ray) and the lobe sample (the first path
 //                segment), and queues both rays;
 //   k_rf_trace   closest hit of every queued ray: a persistent kernel whose
-//                warps draw rays from the queue and walk the tree with the
-//                stage-1 bake's speculative, warp-refilled traversal (stack
-//                in local memory, as the bake's);
+//                warps draw rays from the queue (path segments, then shadow
+//                rays) and walk the tree with the stage-1 bake's walk;
 //   k_rf_shade   consumes a slot's hits (the shadow ray first, then the
 //                path segment), and at a smooth surface queues the vertex's
 //                shadow ray and its next segment together (the BRDF sample
@@ -790,11 +789,12 @@ RfLayout carve_refine(void* base, int64_t N, int64_t P, int waves) {
     L.st.cnt = c.take<uint32_t>(4 * (size_t)(waves + 1));
     // The points are put in Morton order first, in the path state's place (184
     // bytes a sample; the sort takes about 12 a point); calls whose sort does
-    // not fit there (over 190 million points in chunks) keep their own order.
+    // not fit there (over 190 million points in chunks) keep their own order,
+    // and so do calls of a few points, which would wait for the sort's launches.
     L.order_scratch = c.off;
     size_t need = 0;
     L.order = nullptr;
-    if (N < ((int64_t)1 << 31) && fipt_query_order_workspace_size(N, &need) == FIPT_OK && need <= L.order_scratch) {
+    if (N >= 256 && N < ((int64_t)1 << 31) && fipt_query_order_workspace_size(N, &need) == FIPT_OK && need <= L.order_scratch) {
         int32_t* order = c.take<int32_t>((size_t)N);
         L.order = order;
     }

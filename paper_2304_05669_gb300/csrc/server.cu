@@ -7,7 +7,8 @@
 //    FIPT_ERR_BUDGET.  Inputs are copied in on a copy stream.
 //  * The bake loop.  One kernel (k_serve_bake) keeps warps resident on all
 //    block slots of every SM but kRenderBlocksPerSM; they take warp items
-//    (32 points of one chunk, one lobe) from a device counter in the order
+//    (32 points of one chunk, one lobe; 32 / G where G lanes share a pair,
+//    bake_split) from a device counter in the order
 //    the host publishes them and bake each exactly as a standalone
 //    fipt_bake would (chunks keep request-local Philox counters), so a
 //    result is bit-identical alone and in any mix.  The warp that finishes

@@ -549,8 +549,8 @@ __device__ __noinline__ int serve_take_bake(ServeShared* sh, ServeCounters* ctr,
     }
 }
 
-// The server's bake loop: resident warps take bake items (32 points of one
-// chunk, one lobe) in publication order from a device counter with one
+// The server's bake loop: resident warps take bake items (32 / G points of one
+// chunk, one lobe, G = 2^log_g lanes a pair) in publication order from a device counter with one
 // atomicAdd each (no compare-and-swap retries, so thousands of warps do not
 // serialise on the counter), bake each exactly as k_bake would, and count
 // it done; the warp that completes a chunk raises the chunk's flag in
