@@ -671,6 +671,23 @@ __device__ __forceinline__ void better_part(float& v, int& P, int lane_mask) {
     }
 }
 
+// The cheapest split of a subset into {low} with Q and the rest without Q, for
+// Q over the SPLITS proper subsets of rest by falling value (low stands below
+// rest: their union is a sum).  cl and cr: the costs from low and from rest on.
+template <int SPLITS>
+__device__ __forceinline__ void best_split(const float* cl, const float* cr, int rest, float& best, int& bq) {
+    int Q = rest;
+#pragma unroll
+    for (int i = 0; i < SPLITS; ++i) {
+        Q = (Q - 1) & rest;
+        const float v = cl[Q] + cr[-Q];
+        if (v < best) {
+            best = v;
+            bq = Q;
+        }
+    }
+}
+
 // Restructures the treelet rooted at p; all 32 lanes of the warp call it
 // with the same p.  Lane i holds treelet leaf i and internal node i.  The
 // kernel is bound by the instructions it issues, so every part is spread over
@@ -686,7 +703,8 @@ __device__ __forceinline__ void better_part(float& v, int& P, int lane_mask) {
 // A record's d.z holds the pass that last rewrote it.  A treelet none of whose
 // records was rewritten in the last pass or so far in this one is the treelet
 // the last pass found at p and kept, so this pass would keep it too and leaves
-// it: three passes over the floor 5.8 -> 5.1 ms.
+// it: three passes over the floor 5.8 -> 5.1 ms (4.95 with the splits of a
+// subset unrolled and their costs addressed from two bases).
 __device__ void restructure_warp(BvhNode* nodes, int32_t* parent, int32_t* leaf_parent, int p, int pass,
                                  TreeletTables& tb, const uint8_t* subsets, int lane) {
     constexpr unsigned FULL = 0xffffffffu;
@@ -759,17 +777,12 @@ __device__ void restructure_warp(BvhNode* nodes, int32_t* parent, int32_t* leaf_
         for (int i = lane; i < cnt; i += 32) {
             const int S = list[i], low = S & -S, rest = S ^ low;
             float best = inf;
-            int bp = low;
-            for (int Q = (rest - 1) & rest;; Q = (Q - 1) & rest) {
-                const float v = tb.cost[low | Q] + tb.cost[rest ^ Q];
-                if (v < best) {
-                    best = v;
-                    bp = low | Q;
-                }
-                if (Q == 0) break;
-            }
+            int bq = 0;
+            if (k == 3) best_split<3>(tb.cost + low, tb.cost + rest, rest, best, bq);
+            else if (k == 4) best_split<7>(tb.cost + low, tb.cost + rest, rest, best, bq);
+            else best_split<15>(tb.cost + low, tb.cost + rest, rest, best, bq);
             tb.cost[S] = best + tb.area[S];
-            tb.part[S] = (uint8_t)bp;
+            tb.part[S] = (uint8_t)(low | bq);
         }
         __syncwarp();
     }
@@ -777,17 +790,20 @@ __device__ void restructure_warp(BvhNode* nodes, int32_t* parent, int32_t* leaf_
         const int e = lane >> 2;
         const int S = full ^ (1 << e), low = S & -S, rest = S ^ low;
         const int gap = (1 << (e > 1 ? e : 1)) - 1;        // rest holds bits 1.. without bit max(e, 1)
+        const auto spread = [&](int j) { return (j << 1 & gap) | (j << 1 & ~gap) << 1; };
+        const float *cl = tb.cost + low, *cr = tb.cost + rest;
+        const int four = spread(4);
         float best = inf;
-        int bp = low;
+        int bq = 0;
         if (e < m)
-            for (int j = (1 << (m - 2)) - 2 - (lane & 3); j >= 0; j -= 4) {
-                const int t = j << 1, Q = (t & gap) | (t & ~gap) << 1;
-                const float v = tb.cost[low | Q] + tb.cost[rest ^ Q];
+            for (int j = (1 << (m - 2)) - 2 - (lane & 3), Q = spread(j); j >= 0; j -= 4, Q = (Q - four) & rest) {
+                const float v = cl[Q] + cr[-Q];
                 if (v < best) {
                     best = v;
-                    bp = low | Q;
+                    bq = Q;
                 }
             }
+        int bp = low | bq;
         better_part(best, bp, 1);
         better_part(best, bp, 2);
         if (e < m && (lane & 3) == 0) {
