@@ -658,6 +658,7 @@ struct TreeletTables {
     float cost[1 << TREELET];
     uint8_t part[1 << TREELET];
     Box box[TREELET];
+    int size[TREELET];
 };
 
 // The better of two partitions: the lower cost, on a tie the larger subset
@@ -705,7 +706,11 @@ __device__ __forceinline__ void best_split(const float* cl, const float* cr, int
 // the last pass found at p and kept, so this pass would keep it too and leaves
 // it: three passes over the floor 5.8 -> 5.1 ms (4.95 with the splits of a
 // subset unrolled and their costs addressed from two bases).
-__device__ void restructure_warp(BvhNode* nodes, int32_t* parent, int32_t* leaf_parent, int p, int pass,
+//
+// size (the last pass only, else NULL): receives the internal nodes below and
+// at each node, for the depth-first renumbering; the sizes of the treelet's
+// leaves are final when p is reached.
+__device__ void restructure_warp(BvhNode* nodes, int32_t* parent, int32_t* leaf_parent, int32_t* size, int p, int pass,
                                  TreeletTables& tb, const uint8_t* subsets, int lane) {
     constexpr unsigned FULL = 0xffffffffu;
     // lane 0 and 1: p's children
@@ -743,7 +748,16 @@ __device__ void restructure_warp(BvhNode* nodes, int32_t* parent, int32_t* leaf_
         ++m;
     }
     if (m < 3) return;                                     // two leaves have one topology (uniform)
-    if (!__any_sync(FULL, fresh)) return;
+    if (size) {
+        const int below = lane < m && ref >= 0 ? __ldcg(size + ref) : 0;
+        if (lane < m) tb.size[lane] = below;
+        const int all = __reduce_add_sync(FULL, below) + m - 1;
+        if (lane == 0) __stcg(size + p, all);              // whatever the topology
+    }
+    if (!__any_sync(FULL, fresh)) {
+        __syncwarp();
+        return;
+    }
     if (lane < m) tb.box[lane] = box;
     __syncwarp();
     const int full = (1 << m) - 1;
@@ -857,6 +871,11 @@ __device__ void restructure_warp(BvhNode* nodes, int32_t* parent, int32_t* leaf_
         __stcg(reinterpret_cast<int4*>(q + 3), make_int4(r0, r1, pass, 0));
         __stcg(r0 >= 0 ? parent + r0 : leaf_parent + ~r0, inner);
         __stcg(r1 >= 0 ? parent + r1 : leaf_parent + ~r1, inner);
+        if (size && lane > 0) {
+            int n = __popc(mask) - 1;
+            for (int S = mask; S; S &= S - 1) n += tb.size[__ffs(S) - 1];
+            __stcg(size + inner, n);
+        }
         __threadfence();
     }
     __syncwarp();
@@ -869,7 +888,7 @@ constexpr int TL_THREADS = 128;
 // nodes its lanes were second to reach.  A climb longer than any valid
 // tree allows (a corrupt parent chain) stops and raises the step flag.
 __global__ void __launch_bounds__(TL_THREADS, 10)
-k_treelets(BvhNode* nodes, int32_t* parent, int32_t* leaf_parent, int32_t* flags, int64_t T, int pass,
+k_treelets(BvhNode* nodes, int32_t* parent, int32_t* leaf_parent, int32_t* flags, int32_t* size, int64_t T, int pass,
            int32_t* status) {
     constexpr unsigned FULL = 0xffffffffu;
     __shared__ TreeletTables tabs[TL_THREADS / 32];
@@ -899,12 +918,13 @@ k_treelets(BvhNode* nodes, int32_t* parent, int32_t* leaf_parent, int32_t* flags
         if (act) {
             const int2 ch = __ldcg(reinterpret_cast<const int2*>(nodes + p) + 6);
             wide = ch.x >= 0 || ch.y >= 0;
+            if (size && !wide) __stcg(size + p, 1);
         }
         unsigned todo = __ballot_sync(FULL, wide);
         while (todo) {
             const int l = __ffs(todo) - 1;
             todo &= todo - 1;
-            restructure_warp(nodes, parent, leaf_parent, __shfl_sync(FULL, p, l), pass, tb, subsets, lane);
+            restructure_warp(nodes, parent, leaf_parent, size, __shfl_sync(FULL, p, l), pass, tb, subsets, lane);
         }
         if (act) {
             __threadfence();
@@ -1243,11 +1263,12 @@ extern "C" fipt_status fipt_scene_optimize(fipt_scene* s, int32_t passes, fipt_s
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     for (int k = 0; k < passes; ++k) {
         FIPT_CUDA(cudaMemsetAsync(s->flags, 0, sizeof(int32_t) * (size_t)(T - 1), st));
-        FIPT_LAUNCH(k_treelets, grid_for(T, TL_THREADS), TL_THREADS, 0, st, s->nodes, s->parent, s->leaf_parent, s->flags, T,
-                    k + 1, s->ctx->status);
+        FIPT_LAUNCH(k_treelets, grid_for(T, TL_THREADS), TL_THREADS, 0, st, s->nodes, s->parent, s->leaf_parent, s->flags,
+                    k == passes - 1 ? s->scratch : nullptr, T, k + 1, s->ctx->status);
     }
     FIPT_LAUNCHED("treelet restructuring");
     s->restructured = true;
+    s->has_sizes = true;
     return FIPT_OK;
 }
 
@@ -1260,9 +1281,12 @@ extern "C" fipt_status fipt_scene_relayout(fipt_scene* s, fipt_stream stream) {
     int32_t* size = s->scratch;
     int32_t* idx = s->scratch + n;
     int32_t* new_parent = s->scratch + 2 * n;
-    FIPT_CUDA(cudaMemsetAsync(s->flags, 0, sizeof(int32_t) * (size_t)n, st));
-    FIPT_LAUNCH(k_subtree_sizes, grid_for(T, 256), 256, 0, st, s->nodes, s->parent, s->leaf_parent, s->flags, size,
-                T, s->ctx->status);
+    if (!s->has_sizes) {                  // else the last restructuring pass left them
+        FIPT_CUDA(cudaMemsetAsync(s->flags, 0, sizeof(int32_t) * (size_t)n, st));
+        FIPT_LAUNCH(k_subtree_sizes, grid_for(T, 256), 256, 0, st, s->nodes, s->parent, s->leaf_parent, s->flags,
+                    size, T, s->ctx->status);
+    }
+    s->has_sizes = false;                 // of the old numbers
     FIPT_LAUNCH(k_dfs_index, grid_for(n, 256), 256, 0, st, s->nodes, s->parent, size, idx, n, s->ctx->status);
     FIPT_LAUNCH(k_relabel, grid_for(n, 256), 256, 0, st, s->nodes, s->parent, idx, s->nodes_alt, new_parent, n,
                 s->ctx->status);
