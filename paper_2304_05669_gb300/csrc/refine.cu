@@ -216,7 +216,8 @@ struct RfState {
     // records that are used together lie side by side, a slot's pair in one 32-byte sector
     float4* os;         // [2P] origin of the slot's rays (xyz), the triangle they skip (int bits); shadow-ray weights
                         // (rgb), target emitter leaf (int bits)
-    float4* dir;        // [2P] ray 2j: path segment, 2j+1: shadow ray; direction (xyz), t_max
+    float4* dir;        // [2P] ray 2j: path segment, direction (xyz), index of the slot's point (int bits); 2j+1: shadow
+                        // ray, direction, t_max
     int4* hit;          // [2P] t (float bits), leaf (-1: none), original triangle id, front face
     float4* lb;         // [2P] path radiance (rgb), W0; path throughput (rgb), pdf of the last BRDF sample
     float4* cc;         // [2P] sample value for L_d / L_s0 (rgb), W1; for L_s1 (rgb), flags (int bits)
@@ -228,13 +229,11 @@ struct RfState {
 
 struct RfChunk {
     const fipt_query* q;    // the call's queries
-    const int32_t* order;   // the chunk's part of the points' order (NULL: as they are)
-    int64_t p0;             // place of the chunk's first point in that order
+    const int32_t* order;   // [n_pts] order of the chunk's points, during k_rf_gen (NULL: as they are)
+    int64_t p0;             // index of the chunk's first point in the call
     int64_t n_pts;          // points in the chunk
     int64_t P;              // slots: n_pts * per_pt, at most RF_SLOT_CAP
 
-    // index of the chunk's point pc in the call
-    __device__ __forceinline__ int64_t point(uint32_t pc) const { return order ? (int64_t)order[pc] : p0 + pc; }
 };
 
 // A point's samples in order are its spp_d diffuse samples, then spp_s of
@@ -331,7 +330,7 @@ k_rf_gen(SceneView sc, RfChunk C, RefineArgs R, RfState st) {
             uint32_t pc;
             int lobe, s;
             slot_decode((uint32_t)j, R, (uint32_t)C.n_pts, pc, lobe, s);
-            const int64_t pq = C.point(pc);
+            const int64_t pq = C.p0 + (C.order ? (int64_t)C.order[pc] : (int64_t)pc);
             const float2* qp = reinterpret_cast<const float2*>(C.q + pq);
             const float2 q0 = qp[0], q1 = qp[1], q2 = qp[2], q3 = qp[3], q4 = qp[4];
             float3 n = make_float3(q1.y, q2.x, q2.y), wo = make_float3(q3.x, q3.y, q4.x);
@@ -345,6 +344,7 @@ k_rf_gen(SceneView sc, RfChunk C, RefineArgs R, RfState st) {
             // specular terms of points seen at grazing angles are defined as zero
             const bool grazing = lobe > 0 && mu_o <= 1e-2f;
             float4 C0 = make_float4(0.0f, 0.0f, 0.0f, 0.0f), C1 = C0;
+            float3 wp = make_float3(0.0f, 0.0f, 0.0f);              // the first path segment's direction
             uint32_t flags = 0;
             if (!grazing) {
                 float a2 = 0.0f, g1o = 0.0f;
@@ -434,7 +434,7 @@ k_rf_gen(SceneView sc, RfChunk C, RefineArgs R, RfState st) {
                     }
                 }
                 if (ok) {
-                    st.dir[2 * j] = make_float4(wi.x, wi.y, wi.z, FINF);
+                    wp = wi;
                     st.lb[2 * j + 1] = make_float4(1.0f, 1.0f, 1.0f, pb);
                     st.lb[2 * j] = make_float4(0.0f, 0.0f, 0.0f, W0);
                     C0.w = W1;
@@ -444,6 +444,7 @@ k_rf_gen(SceneView sc, RfChunk C, RefineArgs R, RfState st) {
             }
             C1.w = __uint_as_float(flags);
             store_pair(st.cc + 2 * j, C0, C1);
+            st.dir[2 * j] = make_float4(wp.x, wp.y, wp.z, __uint_as_float((uint32_t)pq));
         }
         warp_append(st.act[0], st.cnt + 2, qpath || qshadow, (uint32_t)j);
         warp_append(st.tq[0], st.cnt + 0, qpath, (uint32_t)(2 * j));
@@ -516,11 +517,11 @@ k_rf_trace(SceneView sc, RfState st, int w, int32_t* status, unsigned long long*
                     const float4 o = __ldg(st.os + (rid & ~1)), d = __ldg(st.dir + rid);
                     r = make_ray(o.x, o.y, o.z, d.x, d.y, d.z);
                     skip = __float_as_int(o.w);
-                    best.t = d.w;
+                    shadow = (rid & 1) != 0;
+                    best.t = shadow ? d.w : FINF;      // (a path segment's d.w is its point)
                     best.code = FIPT_DONE;
                     wk.start(sc);
                     if (STATS) ++n_rays;
-                    shadow = (rid & 1) != 0;
                     if (shadow) {                  // settle the target first
                         const int tgt = __float_as_int(__ldg(&st.os[rid | 1].w));
                         const float4 p0 = __ldg(sc.tris + 3 * tgt);
@@ -584,7 +585,6 @@ k_rf_shade(SceneView sc, RfChunk C, RefineArgs R, RfState st, int w) {
             uint32_t pc;
             int lobe, s;
             slot_decode(j, R, (uint32_t)C.n_pts, pc, lobe, s);
-            const uint32_t pid = A.point_base + (uint32_t)C.point(pc);
             float4 C0, C1, LW, BP, O, SW, h0, h1;
             load_pair(st.cc + 2 * j, C0, C1);
             // the slot's other records, loaded together whether or not a ray
@@ -593,6 +593,7 @@ k_rf_shade(SceneView sc, RfChunk C, RefineArgs R, RfState st, int w) {
             load_pair(st.os + 2 * j, O, SW);
             load_pair(reinterpret_cast<const float4*>(st.hit) + 2 * j, h0, h1);
             const float4 D = st.dir[2 * j];
+            const uint32_t pid = A.point_base + __float_as_uint(D.w);
             const int4 h = as_int4(h0), hs = as_int4(h1);
             const uint32_t f_in = __float_as_uint(C1.w);
             uint32_t depth = f_in & F_DEPTH;
@@ -695,7 +696,7 @@ k_rf_shade(SceneView sc, RfChunk C, RefineArgs R, RfState st, int w) {
                         vertex_brdf(M, nv, wv, wi, mu_v, f, pdf, glossy, hh, sin2h);
                         if (pdf > 0.0f) {
                             st.lb[2 * j + 1] = make_float4(BP.x * (f[0] / pdf), BP.y * (f[1] / pdf), BP.z * (f[2] / pdf), pdf);
-                            st.dir[2 * j] = make_float4(wi.x, wi.y, wi.z, FINF);
+                            st.dir[2 * j] = make_float4(wi.x, wi.y, wi.z, D.w);
                             ++depth;
                             flags |= F_PATH;
                             qpath = true;
@@ -732,9 +733,9 @@ k_rf_reduce(RfChunk C, RefineArgs R, RfState st, float* __restrict__ Ld, float* 
     if (t >= C.n_pts * L) return;
     const int lobe = (int)(t / C.n_pts);          // neighbouring threads: neighbouring points
     const int64_t pc = t - lobe * C.n_pts;
-    const int64_t p = C.point((uint32_t)pc);
     const int S = lobe == 0 ? R.A.spp_d : R.A.spp_s;
     const int64_t r0 = lobe == 0 ? 0 : R.A.spp_d + (int64_t)(lobe - 1) * R.A.spp_s;
+    const int64_t p = __float_as_uint(st.dir[2 * slot_of((uint32_t)pc, (uint32_t)r0, R, (uint32_t)C.n_pts)].w);
     float a0 = 0.0f, a1 = 0.0f, a2 = 0.0f, a3 = 0.0f, a4 = 0.0f, a5 = 0.0f;
     float* ps = PER_SAMPLE ? per_sample + (size_t)(p * L + lobe) * R.smax * 6 : nullptr;
     for (int s = 0; s < S; ++s) {
@@ -768,12 +769,10 @@ inline unsigned blocks(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
 struct RfLayout {
     RfState st;
-    int32_t* order;         // [N] the points' order, or NULL
-    size_t order_scratch;   // bytes its sort may use, from the workspace's start
     size_t bytes;
 };
 
-RfLayout carve_refine(void* base, int64_t N, int64_t P, int waves) {
+RfLayout carve_refine(void* base, int64_t P, int waves) {
     Carver c{static_cast<char*>(base), 0};
     RfLayout L;
     L.st.P = (uint32_t)P;
@@ -787,17 +786,6 @@ RfLayout carve_refine(void* base, int64_t N, int64_t P, int waves) {
     L.st.tq[0] = c.take<uint32_t>(2 * P);
     L.st.tq[1] = c.take<uint32_t>(2 * P);
     L.st.cnt = c.take<uint32_t>(4 * (size_t)(waves + 1));
-    // The points are put in Morton order first, in the path state's place (184
-    // bytes a sample; the sort takes about 12 a point); calls whose sort does
-    // not fit there (over 190 million points in chunks) keep their own order,
-    // and so do calls of a few points, which would wait for the sort's launches.
-    L.order_scratch = c.off;
-    size_t need = 0;
-    L.order = nullptr;
-    if (N >= 256 && N < ((int64_t)1 << 31) && fipt_query_order_workspace_size(N, &need) == FIPT_OK && need <= L.order_scratch) {
-        int32_t* order = c.take<int32_t>((size_t)N);
-        L.order = order;
-    }
     L.bytes = (c.off + 255) & ~size_t(255);
     return L;
 }
@@ -825,7 +813,7 @@ extern "C" fipt_status fipt_bake_refine_workspace_size(int64_t N, const fipt_bak
     FIPT_REQUIRE(refine_chunking(prm, N, per_pt, pts, P),
                  "spp_diffuse + K * spp_specular = %lld exceeds %lld samples per point", (long long)per_pt,
                  (long long)RF_SLOT_CAP);
-    *bytes = N == 0 ? 0 : carve_refine(nullptr, N, P, max_depth + 1).bytes;
+    *bytes = N == 0 ? 0 : carve_refine(nullptr, P, max_depth + 1).bytes;
     return FIPT_OK;
 }
 
@@ -852,11 +840,11 @@ extern "C" fipt_status fipt_bake_refine(fipt_scene* s, const fipt_query* q, int6
     FIPT_REQUIRE(fipt_aligned(q, 8) && fipt_aligned(Ld, 4) && fipt_aligned(Ls0, 4) &&
                  fipt_aligned(Ls1, 4) && fipt_aligned(per_sample, 4), "misaligned array");
     const int waves = max_depth + 1;
-    RfLayout lay = carve_refine(nullptr, N, P, waves);
+    RfLayout lay = carve_refine(nullptr, P, waves);
     FIPT_REQUIRE(workspace && fipt_aligned(workspace, 256), "workspace must be 256-byte aligned");
     if (ws_bytes < lay.bytes)
         return fipt_set_error(FIPT_ERR_WORKSPACE, "refine workspace %zu < %zu bytes", ws_bytes, lay.bytes);
-    lay = carve_refine(workspace, N, P, waves);
+    lay = carve_refine(workspace, P, waves);
     FIPT_CUDA(cudaSetDevice(s->ctx->device));
     RefineArgs R;
     R.A.key = make_uint2((uint32_t)prm->seed, (uint32_t)(prm->seed >> 32));
@@ -883,18 +871,26 @@ extern "C" fipt_status fipt_bake_refine(fipt_scene* s, const fipt_query* q, int6
     const unsigned shade_grid = (unsigned)(sms * 8);
     const SceneView sv = s->view();
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (lay.order) {
-        const fipt_status r = fipt_query_order(s, q, N, lay.order, workspace, lay.order_scratch, stream);
-        if (r != FIPT_OK) return r;
-    }
     for (int64_t p0 = 0; p0 < N; p0 += pts) {
         RfChunk C;
         C.q = q;
-        C.order = lay.order ? lay.order + p0 : nullptr;
         C.p0 = p0;
         C.n_pts = N - p0 < pts ? N - p0 : pts;
+        C.order = nullptr;
         C.P = C.n_pts * per_pt;
         FIPT_CUDA(cudaMemsetAsync(lay.st.cnt, 0, sizeof(uint32_t) * 4 * (size_t)(waves + 1), st));
+        // The chunk's points in Morton order, for k_rf_gen alone: it stands where
+        // the second queue comes later, and its sort (12 bytes a point and some
+        // kilobytes) works where the origins and shadow weights do (32 a sample).
+        // A few points do not wait for the sort's launches.
+        size_t need = 0;
+        if (C.n_pts >= 256 && fipt_query_order_workspace_size(C.n_pts, &need) == FIPT_OK &&
+            need <= 2 * sizeof(float4) * (size_t)C.P) {
+            int32_t* order = reinterpret_cast<int32_t*>(lay.st.tq[1]);
+            const fipt_status r = fipt_query_order(s, q + p0, C.n_pts, order, lay.st.os, need, stream);
+            if (r != FIPT_OK) return r;
+            C.order = order;
+        }
         const unsigned gen_grid = blocks(C.P, RF_SHADE_THREADS) < shade_grid ? blocks(C.P, RF_SHADE_THREADS) : shade_grid;
         FIPT_LAUNCH(k_rf_gen, gen_grid, RF_SHADE_THREADS, 0, st, sv, C, R, lay.st);
         for (int w = 0; w < waves; ++w) {
