@@ -747,14 +747,15 @@ __device__ void restructure_warp(BvhNode* nodes, int32_t* parent, int32_t* leaf_
         if (lane == best || lane == m) take_child(n, lane == m);
         ++m;
     }
-    if (m < 3) return;                                     // two leaves have one topology (uniform)
     if (size) {
         const int below = lane < m && ref >= 0 ? __ldcg(size + ref) : 0;
         if (lane < m) tb.size[lane] = below;
         const int all = __reduce_add_sync(FULL, below) + m - 1;
         if (lane == 0) __stcg(size + p, all);              // whatever the topology
     }
-    if (!__any_sync(FULL, fresh)) {
+    // nothing changed, or two leaves: one topology (internal leaves whose box has no area to compare, infinity times
+    // zero, stay closed)
+    if (m < 3 || !__any_sync(FULL, fresh)) {
         __syncwarp();
         return;
     }
