@@ -33,21 +33,38 @@ k_trace(SceneView sc, const float* __restrict__ orig, const float* __restrict__ 
 // A warp looks through a tile of 8 x 4 pixels (2^log_tw x 32 / 2^log_tw),
 // whose rays walk the tree more alike than those of 32 pixels of a row (24
 // views of 640 x 416 in the room: 820 -> 776 us).  Lanes past the image's
-// edges have no ray.
+// edges have no ray, and views too small to fill their tiles by CAMERA_FILL pixels
+// take 32 pixels in order instead, across rows and views, with log_tw < 0 (1.5 M
+// pixels of the room in tiles / in order, us: 97 x 131 with 29.6 pixels a tile
+// 292 / 305, 65 x 49 with 27.2 359 / 357, 41 x 37 with 25.3 376 / 363, 17 x 17 with
+// 19.3 456 / 386, 4 x 4 with 16 655 / 472, 1 x 1 3,831 / 417).
+constexpr int CAMERA_FILL = 28;      // pixels per tile, on average, from which there are tiles
+
 __global__ void __launch_bounds__(TRACE_THREADS, TRACE_MINB)
-k_camera(SceneView sc, const float* __restrict__ cams, int W, int H, int log_tw, int tiles_x, int tiles_y, int64_t tiles,
-         fipt_query* __restrict__ out, int32_t* __restrict__ valid, int32_t* status) {
-    const int64_t tile = (blockIdx.x * (int64_t)TRACE_THREADS + threadIdx.x) >> 5;
-    if (tile >= tiles) return;                             // whole warp
+k_camera(SceneView sc, const float* __restrict__ cams, int W, int H, int log_tw, int tiles_x, int tiles_y, int64_t warps,
+         int64_t P, fipt_query* __restrict__ out, int32_t* __restrict__ valid, int32_t* status) {
+    const int64_t warp = (blockIdx.x * (int64_t)TRACE_THREADS + threadIdx.x) >> 5;
+    if (warp >= warps) return;                             // whole warp
     const int lane = threadIdx.x & 31;
-    const int64_t row = tile / tiles_x;                    // tile rows, view after view
-    const int v = (int)(row / tiles_y);
-    int i = ((int)(tile - row * tiles_x) << log_tw) + (lane & ((1 << log_tw) - 1));
-    int j = ((int)(row - (int64_t)v * tiles_y) << (5 - log_tw)) + (lane >> log_tw);
-    const bool on = i < W && j < H;
-    i = min(i, W - 1);
-    j = min(j, H - 1);
-    const int64_t p = ((int64_t)v * H + j) * W + i;
+    int v, i, j, p;                                        // p < P < 2^31
+    bool on;
+    if (log_tw < 0) {                                      // 32 pixels in order
+        on = warp * 32 + lane < P;
+        p = (int)(on ? warp * 32 + lane : P - 1);
+        const int row = p / W;
+        i = p - row * W;
+        v = row / H;
+        j = row - v * H;
+    } else {
+        const int64_t row = warp / tiles_x;                // tile rows, view after view
+        v = (int)(row / tiles_y);
+        i = ((int)(warp - row * tiles_x) << log_tw) + (lane & ((1 << log_tw) - 1));
+        j = ((int)(row - (int64_t)v * tiles_y) << (5 - log_tw)) + (lane >> log_tw);
+        on = i < W && j < H;
+        i = min(i, W - 1);
+        j = min(j, H - 1);
+        p = (v * H + j) * W + i;
+    }
     const float* c = cams + 10 * v;
     float fx = c[3], fy = c[4], fz = c[5];
     const float fl = 1.0f / sqrtf(fx * fx + fy * fy + fz * fz);
@@ -789,8 +806,10 @@ extern "C" fipt_status fipt_camera_queries(fipt_scene* s, const float* cams, int
     const int tw = 1 << log_tw, th = 32 >> log_tw;
     const int tiles_x = (int)(((int64_t)W + tw - 1) / tw), tiles_y = (int)(((int64_t)H + th - 1) / th);
     const int64_t tiles = (int64_t)nViews * tiles_x * tiles_y;
-    FIPT_LAUNCH(k_camera, blocks(tiles * 32, TRACE_THREADS), TRACE_THREADS, 0, static_cast<cudaStream_t>(stream),
-                s->view(), cams, W, H, log_tw, tiles_x, tiles_y, tiles, out, valid, s->ctx->status);
+    const bool tiled = P >= tiles * CAMERA_FILL;
+    const int64_t warps = tiled ? tiles : (P + 31) / 32;
+    FIPT_LAUNCH(k_camera, blocks(warps * 32, TRACE_THREADS), TRACE_THREADS, 0, static_cast<cudaStream_t>(stream),
+                s->view(), cams, W, H, tiled ? log_tw : -1, tiles_x, tiles_y, warps, P, out, valid, s->ctx->status);
     FIPT_LAUNCHED("camera_queries");
     return FIPT_OK;
 }
