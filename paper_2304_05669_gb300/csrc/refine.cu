@@ -216,8 +216,7 @@ struct RfState {
     // records that are used together lie side by side, a slot's pair in one 32-byte sector
     float4* os;         // [2P] origin of the slot's rays (xyz), the triangle they skip (int bits); shadow-ray weights
                         // (rgb), target emitter leaf (int bits)
-    float4* dir;        // [2P] ray 2j: path segment, direction (xyz), index of the slot's point (int bits); 2j+1: shadow
-                        // ray, direction, t_max
+    float4* dir;        // [2P] ray 2j: path segment, 2j+1: shadow ray; direction (xyz), t_max
     int4* hit;          // [2P] t (float bits), leaf (-1: none), original triangle id, front face
     float4* lb;         // [2P] path radiance (rgb), W0; path throughput (rgb), pdf of the last BRDF sample
     float4* cc;         // [2P] sample value for L_d / L_s0 (rgb), W1; for L_s1 (rgb), flags (int bits)
@@ -228,22 +227,25 @@ struct RfState {
 };
 
 struct RfChunk {
-    const fipt_query* q;    // the call's queries
-    const int32_t* order;   // [n_pts] order of the chunk's points, during k_rf_gen (NULL: as they are)
-    int64_t p0;             // index of the chunk's first point in the call
+    const fipt_query* q;    // the chunk's first query
+    int64_t p0;             // index of that query in the call
     int64_t n_pts;          // points in the chunk
     int64_t P;              // slots: n_pts * per_pt, at most RF_SLOT_CAP
-
 };
 
 // A point's samples in order are its spp_d diffuse samples, then spp_s of
 // each roughness level.  Slots hold G = 2^log_g consecutive samples of a point
-// side by side, point after point in the Morton order of their positions, so
-// that a warp's first rays leave one point through neighbouring strata and walk
-// the tree alike.  The samples left over by G come last, a point's together.
-// 131,072 points of the room x 32 samples x 7 lobes: 43.4 ms in pixel order
-// with a sample of 32 points a warp, 42.7 in Morton order, 42.4 / 42.2 / 41.9 /
-// 41.7 / 41.4 with 2 / 4 / 8 / 16 / 32 samples together.
+// side by side, point after point, so that a warp's first rays leave one point
+// through neighbouring strata and walk the tree alike.  The samples left over by
+// G come last, a point's together.  131,072 points of the room x 32 samples x 7
+// lobes, points in Morton order: 42.7 ms with a sample of 32 points a warp, 42.4 /
+// 42.2 / 41.9 / 41.7 / 41.4 with 2 / 4 / 8 / 16 / 32 samples together.  With the
+// samples together the points' own order hardly matters, and they are taken as
+// they come: sorting a chunk's points first cost 20 us up to 8,192 of them and 65
+// above (in all, sorted / as they come: Cornell box, 9,000 points x 2 samples x 7
+// lobes 0.397 / 0.311 ms; room in pixel order, 9,000 x 8 1.66 / 1.57, 131,072 x 8
+// 10.61 / 10.44, x 32 39.6 / 39.3), and gained only for many points in random order
+// with few samples each (131,072 x 8 10.65 / 10.84, 400,000 x 2 8.64 / 9.01).
 __device__ __forceinline__ uint32_t slot_of(uint32_t pc, uint32_t r, const RefineArgs& R, uint32_t n_pts) {
     const uint32_t lg = (uint32_t)R.log_g, whole = (uint32_t)R.per_pt >> lg << lg;
     if (r < whole) return (((r >> lg) * n_pts + pc) << lg) + (r & ((1u << lg) - 1u));
@@ -330,8 +332,7 @@ k_rf_gen(SceneView sc, RfChunk C, RefineArgs R, RfState st) {
             uint32_t pc;
             int lobe, s;
             slot_decode((uint32_t)j, R, (uint32_t)C.n_pts, pc, lobe, s);
-            const int64_t pq = C.p0 + (C.order ? (int64_t)C.order[pc] : (int64_t)pc);
-            const float2* qp = reinterpret_cast<const float2*>(C.q + pq);
+            const float2* qp = reinterpret_cast<const float2*>(C.q + pc);
             const float2 q0 = qp[0], q1 = qp[1], q2 = qp[2], q3 = qp[3], q4 = qp[4];
             float3 n = make_float3(q1.y, q2.x, q2.y), wo = make_float3(q3.x, q3.y, q4.x);
             {
@@ -344,7 +345,6 @@ k_rf_gen(SceneView sc, RfChunk C, RefineArgs R, RfState st) {
             // specular terms of points seen at grazing angles are defined as zero
             const bool grazing = lobe > 0 && mu_o <= 1e-2f;
             float4 C0 = make_float4(0.0f, 0.0f, 0.0f, 0.0f), C1 = C0;
-            float3 wp = make_float3(0.0f, 0.0f, 0.0f);              // the first path segment's direction
             uint32_t flags = 0;
             if (!grazing) {
                 float a2 = 0.0f, g1o = 0.0f;
@@ -357,7 +357,7 @@ k_rf_gen(SceneView sc, RfChunk C, RefineArgs R, RfState st) {
                     a2 = al * al;
                     g1o = smith_g1(mu_o, a2);
                 }
-                const uint32_t pid = A.point_base + (uint32_t)pq;
+                const uint32_t pid = A.point_base + (uint32_t)(C.p0 + pc);
                 const float ox = q0.x + eps * n.x, oy = q0.y + eps * n.y, oz = q1.x + eps * n.z;
                 st.os[2 * j] = make_float4(ox, oy, oz, q4.y);         // q4.y: the query's triangle
                 if (mis) {                                          // emitter sample at x
@@ -434,7 +434,7 @@ k_rf_gen(SceneView sc, RfChunk C, RefineArgs R, RfState st) {
                     }
                 }
                 if (ok) {
-                    wp = wi;
+                    st.dir[2 * j] = make_float4(wi.x, wi.y, wi.z, FINF);
                     st.lb[2 * j + 1] = make_float4(1.0f, 1.0f, 1.0f, pb);
                     st.lb[2 * j] = make_float4(0.0f, 0.0f, 0.0f, W0);
                     C0.w = W1;
@@ -444,7 +444,6 @@ k_rf_gen(SceneView sc, RfChunk C, RefineArgs R, RfState st) {
             }
             C1.w = __uint_as_float(flags);
             store_pair(st.cc + 2 * j, C0, C1);
-            st.dir[2 * j] = make_float4(wp.x, wp.y, wp.z, __uint_as_float((uint32_t)pq));
         }
         warp_append(st.act[0], st.cnt + 2, qpath || qshadow, (uint32_t)j);
         warp_append(st.tq[0], st.cnt + 0, qpath, (uint32_t)(2 * j));
@@ -518,7 +517,7 @@ k_rf_trace(SceneView sc, RfState st, int w, int32_t* status, unsigned long long*
                     r = make_ray(o.x, o.y, o.z, d.x, d.y, d.z);
                     skip = __float_as_int(o.w);
                     shadow = (rid & 1) != 0;
-                    best.t = shadow ? d.w : FINF;      // (a path segment's d.w is its point)
+                    best.t = d.w;
                     best.code = FIPT_DONE;
                     wk.start(sc);
                     if (STATS) ++n_rays;
@@ -593,7 +592,7 @@ k_rf_shade(SceneView sc, RfChunk C, RefineArgs R, RfState st, int w) {
             load_pair(st.os + 2 * j, O, SW);
             load_pair(reinterpret_cast<const float4*>(st.hit) + 2 * j, h0, h1);
             const float4 D = st.dir[2 * j];
-            const uint32_t pid = A.point_base + __float_as_uint(D.w);
+            const uint32_t pid = A.point_base + (uint32_t)(C.p0 + pc);
             const int4 h = as_int4(h0), hs = as_int4(h1);
             const uint32_t f_in = __float_as_uint(C1.w);
             uint32_t depth = f_in & F_DEPTH;
@@ -696,7 +695,7 @@ k_rf_shade(SceneView sc, RfChunk C, RefineArgs R, RfState st, int w) {
                         vertex_brdf(M, nv, wv, wi, mu_v, f, pdf, glossy, hh, sin2h);
                         if (pdf > 0.0f) {
                             st.lb[2 * j + 1] = make_float4(BP.x * (f[0] / pdf), BP.y * (f[1] / pdf), BP.z * (f[2] / pdf), pdf);
-                            st.dir[2 * j] = make_float4(wi.x, wi.y, wi.z, D.w);
+                            st.dir[2 * j] = make_float4(wi.x, wi.y, wi.z, FINF);
                             ++depth;
                             flags |= F_PATH;
                             qpath = true;
@@ -735,7 +734,7 @@ k_rf_reduce(RfChunk C, RefineArgs R, RfState st, float* __restrict__ Ld, float* 
     const int64_t pc = t - lobe * C.n_pts;
     const int S = lobe == 0 ? R.A.spp_d : R.A.spp_s;
     const int64_t r0 = lobe == 0 ? 0 : R.A.spp_d + (int64_t)(lobe - 1) * R.A.spp_s;
-    const int64_t p = __float_as_uint(st.dir[2 * slot_of((uint32_t)pc, (uint32_t)r0, R, (uint32_t)C.n_pts)].w);
+    const int64_t p = C.p0 + pc;
     float a0 = 0.0f, a1 = 0.0f, a2 = 0.0f, a3 = 0.0f, a4 = 0.0f, a5 = 0.0f;
     float* ps = PER_SAMPLE ? per_sample + (size_t)(p * L + lobe) * R.smax * 6 : nullptr;
     for (int s = 0; s < S; ++s) {
@@ -873,24 +872,11 @@ extern "C" fipt_status fipt_bake_refine(fipt_scene* s, const fipt_query* q, int6
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     for (int64_t p0 = 0; p0 < N; p0 += pts) {
         RfChunk C;
-        C.q = q;
+        C.q = q + p0;
         C.p0 = p0;
         C.n_pts = N - p0 < pts ? N - p0 : pts;
-        C.order = nullptr;
         C.P = C.n_pts * per_pt;
         FIPT_CUDA(cudaMemsetAsync(lay.st.cnt, 0, sizeof(uint32_t) * 4 * (size_t)(waves + 1), st));
-        // The chunk's points in Morton order, for k_rf_gen alone: it stands where
-        // the second queue comes later, and its sort (12 bytes a point and some
-        // kilobytes) works where the origins and shadow weights do (32 a sample).
-        // A few points do not wait for the sort's launches.
-        size_t need = 0;
-        if (C.n_pts >= 256 && fipt_query_order_workspace_size(C.n_pts, &need) == FIPT_OK &&
-            need <= 2 * sizeof(float4) * (size_t)C.P) {
-            int32_t* order = reinterpret_cast<int32_t*>(lay.st.tq[1]);
-            const fipt_status r = fipt_query_order(s, q + p0, C.n_pts, order, lay.st.os, need, stream);
-            if (r != FIPT_OK) return r;
-            C.order = order;
-        }
         const unsigned gen_grid = blocks(C.P, RF_SHADE_THREADS) < shade_grid ? blocks(C.P, RF_SHADE_THREADS) : shade_grid;
         FIPT_LAUNCH(k_rf_gen, gen_grid, RF_SHADE_THREADS, 0, st, sv, C, R, lay.st);
         for (int w = 0; w < waves; ++w) {
