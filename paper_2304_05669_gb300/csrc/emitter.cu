@@ -210,13 +210,33 @@ k_emit_classify(const float* __restrict__ alpha, int64_t T, int n, double thr,
 // over the lanes.  Adding a term is one 32 x 32 + 64-bit multiply-add by a
 // power of two.  A warp takes 32 rows, so that the FP64 division of each is a
 // lane's.  100 samples on 2,045,464 triangles: 309 us staged (ALU-bound on
-// 64-bit shifts, 17 % of the warps) -> 186 us, 121 at the copy rate.
+// 64-bit shifts, 17 % of the warps) -> 186 us, 121 at the copy rate.  The kernel
+// takes the same time for shorter rows, so they stay staged below ROW_MIN: 4 / 20 /
+// 40 / 48 / 52 / 56 / 72 samples on 2,000,000 triangles, 55 / 150 / 158 / 199 / 220 /
+// 241 / 238 us staged, 173 to 180 here (on 176,000: 40 samples 16.8 / 20.6, 52 20.3 /
+// 20.6, 56 21.1 / 20.6).  Rows outside the exact range are added up in order at the
+// end, a row a lane like the divisions (100 samples 2^60 apart on 176,000
+// triangles: 298 us by one of a row's lanes at a time, 98 staged, 84 here).
 constexpr int ROW_THREADS = 128;
 constexpr int ROW_LANES = 4;
 constexpr int ROW_V = 8;
 constexpr int ROW_MAX = 4 * ROW_V * ROW_LANES;
+constexpr int ROW_MIN = 52;
 
-__global__ void __launch_bounds__(ROW_THREADS)
+// A row's sum in sample order (a call, so that its registers do not cost the rows in the exact range warps).
+__device__ __noinline__ double sum_row(const float4* __restrict__ row, int n4) {
+    double s = 0.0;
+    for (int i = 0; i < n4; ++i) {
+        const float4 v = __ldg(row + i);
+        s += (double)v.x;
+        s += (double)v.y;
+        s += (double)v.z;
+        s += (double)v.w;
+    }
+    return s;
+}
+
+__global__ void __launch_bounds__(ROW_THREADS, 10)
 k_emit_classify_rows(const float4* __restrict__ alpha, int64_t T, int n, double thr, double* __restrict__ mean,
                      uint8_t* __restrict__ flag) {
     constexpr unsigned FULL = 0xffffffffu;
@@ -248,7 +268,7 @@ k_emit_classify_rows(const float4* __restrict__ alpha, int64_t T, int n, double 
             rg.lo = min(rg.lo, __shfl_xor_sync(FULL, rg.lo, o));
             rg.hi = max(rg.hi, __shfl_xor_sync(FULL, rg.hi, o));
         }
-        double s;
+        double s = __longlong_as_double(-1);               // marks a row outside the exact range
         if (!rg.special() && rg.exact_for(n)) {
             const int emin = rg.emin();
             long long acc = 0;
@@ -264,11 +284,6 @@ k_emit_classify_rows(const float4* __restrict__ alpha, int64_t T, int n, double 
 #pragma unroll
             for (int o = 1; o < ROW_LANES; o <<= 1) acc += __shfl_xor_sync(group, acc, o);
             s = fipt_exact::scaled_double(acc, emin);
-        } else {
-            s = 0.0;
-            const float* x = reinterpret_cast<const float*>(row);
-            if (c == 0)
-                for (int j = 0; j < n; ++j) s += (double)x[j];
         }
         __syncwarp();
         const double got = __shfl_sync(FULL, s, lane % (32 / ROW_LANES) * ROW_LANES);
@@ -276,6 +291,7 @@ k_emit_classify_rows(const float4* __restrict__ alpha, int64_t T, int n, double 
     }
     const int64_t t = t0 + lane;
     if (t >= T) return;
+    if (__double2hiint(mine) == -1) mine = sum_row(alpha + t * n4, n4);
     const double m = mine / (double)n;
     if (mean) mean[t] = m;
     flag[t] = m > thr ? 1 : 0;
@@ -604,7 +620,7 @@ extern "C" fipt_status fipt_emitter_classify(const float* alpha, int64_t T, int3
     FIPT_REQUIRE(!mean_alpha || fipt_aligned(mean_alpha, 8), "mean_alpha misaligned");
     const unsigned nb = blocks(T, CLS_THREADS);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (n_per_tri % 4 == 0 && n_per_tri <= ROW_MAX && fipt_aligned(alpha, 16))
+    if (n_per_tri % 4 == 0 && n_per_tri >= ROW_MIN && n_per_tri <= ROW_MAX && fipt_aligned(alpha, 16))
         FIPT_LAUNCH(k_emit_classify_rows, blocks(T, ROW_THREADS), ROW_THREADS, 0, st,
                     reinterpret_cast<const float4*>(alpha), T, n_per_tri, (double)threshold, mean_alpha, is_emitter);
     else if (n_per_tri <= CLS_STAGE_N)
