@@ -68,14 +68,18 @@ __global__ void k_debug_divide(DivN d, const uint32_t* __restrict__ i, int64_t c
 // rate): 1,062 us with a point per thread and float4 stores, 821 / 726 with 4 per
 // thread in blocks of 256 / 128, 690 / 670 with 8, 640 with
 // 16 in blocks of 128.
+// With few samples per triangle (under PTS_MANY) many of a thread's samples wait
+// for another triangle's records, one after the other, so a thread takes 4: 1 / 4 /
+// 8 / 14 / 16 / 24 samples on 2,045,464 triangles 29 / 45 / 75 / 123 / 135 / 192 us,
+// with 16 a thread 74 / 80 / 89 / 144 / 115 / 162.
 constexpr int PTS_THREADS = 128;
-constexpr int PTS_PER = 16;
-constexpr int PTS_BLOCK = PTS_THREADS * PTS_PER;
+constexpr int PTS_MANY = 16;
 
-template <class IDX>
+template <class IDX, int PTS_PER>
 __global__ void __launch_bounds__(PTS_THREADS)
 k_emit_points(const float4* __restrict__ tris, const int32_t* __restrict__ inv, int64_t T, int n, DivN dn,
               uint2 key, uint32_t rid, float* __restrict__ x) {
+    constexpr int PTS_BLOCK = PTS_THREADS * PTS_PER;
     __shared__ __align__(128) float sb[3 * PTS_BLOCK];
     const int64_t total = T * n;
     const int64_t base = (int64_t)blockIdx.x * PTS_BLOCK;
@@ -600,12 +604,18 @@ extern "C" fipt_status fipt_emitter_sample_points(fipt_scene* s, uint64_t seed, 
     const int64_t n = s->T * n_per_tri;
     const uint2 key = make_uint2((uint32_t)seed, (uint32_t)(seed >> 32));
     const DivN dn = div_by((uint32_t)n_per_tri);
-    if (n < ((int64_t)1 << 32))
-        FIPT_LAUNCH(k_emit_points<uint32_t>, blocks(n, PTS_BLOCK), PTS_THREADS, 0,
-                    static_cast<cudaStream_t>(stream), s->tris, s->inv, s->T, n_per_tri, dn, key, request_id, x);
-    else
-        FIPT_LAUNCH(k_emit_points<int64_t>, blocks(n, PTS_BLOCK), PTS_THREADS, 0,
-                    static_cast<cudaStream_t>(stream), s->tris, s->inv, s->T, n_per_tri, dn, key, request_id, x);
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+#define FIPT_POINTS(IDX, PER)                                                                                          \
+    FIPT_LAUNCH((k_emit_points<IDX, PER>), blocks(n, PTS_THREADS * PER), PTS_THREADS, 0, st, s->tris, s->inv, s->T,    \
+                n_per_tri, dn, key, request_id, x)
+    if (n < ((int64_t)1 << 32)) {
+        if (n_per_tri >= PTS_MANY) FIPT_POINTS(uint32_t, 16);
+        else FIPT_POINTS(uint32_t, 4);
+    } else {
+        if (n_per_tri >= PTS_MANY) FIPT_POINTS(int64_t, 16);
+        else FIPT_POINTS(int64_t, 4);
+    }
+#undef FIPT_POINTS
     FIPT_LAUNCHED("emitter sample points");
     return FIPT_OK;
 }
