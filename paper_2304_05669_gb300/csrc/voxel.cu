@@ -153,99 +153,175 @@ k_vox_compact(const uint32_t* __restrict__ keys, int64_t P, const uint32_t* __re
 }
 
 constexpr int MEAN_THREADS = 128;
-constexpr int MEAN_LANES = 8;    // lanes per run
+constexpr int MEAN_LANES = 8;    // lanes per run where the runs are long
+constexpr int MEAN_SHORT = 8;    // pixels per run, on average, from which they are
 constexpr int VU = 4;            // pixels a lane takes at a time
 
-// MEAN_LANES lanes per voxel run, which take its pixels MEAN_LANES * VU at a
-// time, the next pixel indices loading while this group's radiance is
-// fetched.  Each channel's FP64 sum in pixel order is carried exactly in
-// integers (exact_sum.cuh), which add up in any order: a lane keeps its own
-// smallest exponent (over the three channels together) and rescales its sums
-// when a group brings a smaller one, and the lanes' sums meet at the run's
-// smallest.  A run that leaves the exact range is summed again with FP64
-// additions in pixel order.  The kernel is bound by its longest runs (4,194,304
-// pixels of the room in 256^3 cells: 210 us with a lane per run, 17 % of the
-// warps active -> 62 us), then by the gathers; lanes 0 to 2 divide a channel
-// each.
-__global__ void __launch_bounds__(MEAN_THREADS)
-k_vox_means(const uint32_t* __restrict__ keys, const uint32_t* __restrict__ pix, const uint32_t* __restrict__ heads,
-            const uint32_t* __restrict__ nhead, const float* __restrict__ L, float4* __restrict__ grid) {
+// The sums of one run per LANES lanes (lane c of them, run [j0, j1) of count
+// pixels, the same for all), which take its pixels LANES * VU at a time, the next
+// pixel indices loading while this group's radiance is fetched.  Each channel's
+// FP64 sum in pixel order is carried exactly in integers (exact_sum.cuh), which
+// add up in any order: a lane keeps its own smallest exponent (over the three
+// channels together) and rescales its sums when a group brings a smaller one,
+// and the lanes' sums meet at the run's smallest, emin.  False where the run
+// leaves the exact range.  The warp's lanes call it together.
+template <int LANES>
+__device__ __forceinline__ bool run_sums(const uint32_t* __restrict__ pix, const float* __restrict__ L, uint32_t j0,
+                                         uint32_t j1, int c, long long (&acc)[3], int& emin) {
     constexpr unsigned FULL = 0xffffffffu;
-    constexpr int STEP = MEAN_LANES * VU;
-    const int64_t nh = *nhead;
-    const int c = threadIdx.x % MEAN_LANES;
-    const int64_t runs = (int64_t)gridDim.x * MEAN_THREADS / MEAN_LANES;
-    // the lanes of a warp go round together (runs past nh are empty)
-    for (int64_t h = (blockIdx.x * (int64_t)MEAN_THREADS + threadIdx.x) / MEAN_LANES;
-         __any_sync(FULL, h < nh); h += runs) {
-        const int64_t j0 = h < nh ? heads[h] : 0, j1 = h < nh ? heads[h + 1] : 0;
-        const int64_t count = j1 - j0;
-        long long acc[3] = {0, 0, 0};
-        int emin = fipt_exact::EMPTY_EMIN;
-        fipt_exact::Range run;
-        bool ok = fipt_exact::spread_limit(count) >= 0;
-        uint32_t qn[VU];
+    constexpr int STEP = LANES * VU;
+    const int count = (int)(j1 - j0);                        // under 2^31 pixels
+#pragma unroll
+    for (int k = 0; k < 3; ++k) acc[k] = 0;
+    emin = fipt_exact::EMPTY_EMIN;
+    fipt_exact::Range run;
+    bool ok = fipt_exact::spread_limit(count) >= 0;
+    uint32_t qn[VU];
+#pragma unroll
+    for (int u = 0; u < VU; ++u) {
+        const uint32_t e = j0 + c + u * LANES;
+        qn[u] = e < j1 ? pix[e] : 0u;
+    }
+    for (uint32_t e = j0 + c; e < j1 && ok; e += STEP) {
+        float v[VU][3];
 #pragma unroll
         for (int u = 0; u < VU; ++u) {
-            const int64_t e = j0 + c + u * MEAN_LANES;
-            qn[u] = e < j1 ? pix[e] : 0u;
+            const int64_t q = 3 * (int64_t)qn[u];
+            const bool in = e + u * LANES < j1;
+            v[u][0] = in ? L[q] : 0.0f;
+            v[u][1] = in ? L[q + 1] : 0.0f;
+            v[u][2] = in ? L[q + 2] : 0.0f;
         }
-        for (int64_t e = j0 + c; e < j1 && ok; e += STEP) {
-            float v[VU][3];
 #pragma unroll
-            for (int u = 0; u < VU; ++u) {
-                const int64_t q = 3 * (int64_t)qn[u];
-                const bool in = e + u * MEAN_LANES < j1;
-                v[u][0] = in ? L[q] : 0.0f;
-                v[u][1] = in ? L[q + 1] : 0.0f;
-                v[u][2] = in ? L[q + 2] : 0.0f;
-            }
+        for (int u = 0; u < VU; ++u) {
+            const uint32_t x = e + STEP + u * LANES;
+            qn[u] = x < j1 ? pix[x] : 0u;
+        }
 #pragma unroll
-            for (int u = 0; u < VU; ++u) {
-                const int64_t x = e + STEP + u * MEAN_LANES;
-                qn[u] = x < j1 ? pix[x] : 0u;
-            }
+        for (int u = 0; u < VU; ++u)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) run.note(v[u][k]);
+        const int em = run.emin();
+        if (em < emin) {            // from EMPTY_EMIN the sums are still 0
+            const int sh = min(emin - em, 63);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) acc[k] = (long long)((unsigned long long)acc[k] << sh);
+            emin = em;
+        }
+        ok = !run.special() && run.exact_for(count);
+        if (ok) {
 #pragma unroll
             for (int u = 0; u < VU; ++u)
 #pragma unroll
-                for (int k = 0; k < 3; ++k) run.note(v[u][k]);
-            const int em = run.emin();
-            if (em < emin) {            // from EMPTY_EMIN the sums are still 0
-                const int sh = min(emin - em, 63);
+                for (int k = 0; k < 3; ++k) acc[k] = fipt_exact::add_term(acc[k], v[u][k], emin);
+        }
+    }
+    if (LANES == 1) return ok;
+    // the run's range and sums over its lanes
 #pragma unroll
-                for (int k = 0; k < 3; ++k) acc[k] = (long long)((unsigned long long)acc[k] << sh);
-                emin = em;
-            }
-            ok = !run.special() && run.exact_for(count);
+    for (int o = 1; o < LANES; o <<= 1) {
+        run.lo = min(run.lo, __shfl_xor_sync(FULL, run.lo, o));
+        run.hi = max(run.hi, __shfl_xor_sync(FULL, run.hi, o));
+    }
+    const unsigned lanes = ((1u << LANES) - 1u) << (threadIdx.x & 31 & ~(LANES - 1));
+    ok = (__ballot_sync(FULL, ok) & lanes) == lanes && !run.special() && run.exact_for(count);
+    const int sh = ok ? emin - run.emin() : 0;             // 0 to 29 where the lane has a nonzero value
+    emin = run.emin();
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        acc[k] = acc[k] == 0 ? 0 : (long long)((unsigned long long)acc[k] << min(sh, 63));
+#pragma unroll
+        for (int o = 1; o < LANES; o <<= 1) acc[k] += __shfl_xor_sync(FULL, acc[k], o);
+    }
+    return ok;
+}
+
+// Means of the runs.  Long runs take MEAN_LANES lanes each, as the kernel is
+// bound by its longest ones (4,194,304 pixels of the room in 256^3 cells, 14 a
+// run: 210 us with a lane per run, 17 % of the warps active -> 62 us), then by
+// the gathers.  Where a run has under MEAN_SHORT pixels on average most of those
+// lanes would idle: a warp takes 32 runs, a lane each, and then the long ones among
+// them as before (4,194,304 points in 256^3 cells, 1.1 a run: the whole call 906 us
+// with MEAN_LANES for all, 548 with a lane for all, 494).
+//
+// Runs outside the exact range are listed by their block, which then adds up
+// ten of them a warp, every lane a channel of one, in FP64 in pixel order
+// (4,194,304 points in 64^3 cells, all outside it: 403 us with a lane a run, 480
+// with three lanes of MEAN_LANES, 400).  There is a thread per pixel, so a warp
+// for every `per` runs.
+__global__ void __launch_bounds__(MEAN_THREADS)
+k_vox_means(const uint32_t* __restrict__ keys, const uint32_t* __restrict__ pix, const uint32_t* __restrict__ heads,
+            const uint32_t* __restrict__ nhead, int64_t P, const float* __restrict__ L, float4* __restrict__ grid) {
+    constexpr unsigned FULL = 0xffffffffu;
+    __shared__ uint2 wide[MEAN_THREADS];                   // [j0, j1) of the block's runs outside the exact range
+    __shared__ int n_wide;
+    const int nh = (int)*nhead;
+    const int per = P >= MEAN_SHORT * (int64_t)nh ? 32 / MEAN_LANES : 32;      // runs a warp takes
+    if ((int64_t)blockIdx.x * (MEAN_THREADS / 32) * per >= nh) return;         // whole block
+    if (threadIdx.x == 0) n_wide = 0;
+    __syncthreads();
+    const int lane = threadIdx.x & 31, c = lane % MEAN_LANES;
+    const int h = (int)(blockIdx.x * (MEAN_THREADS / 32) + (threadIdx.x >> 5)) * per + (per == 32 ? lane : lane / MEAN_LANES);
+    const uint32_t j0 = h < nh ? heads[h] : 0, j1 = h < nh ? heads[h + 1] : 0;     // empty past nh
+    uint32_t r0 = j0, r1 = j1;
+    unsigned todo = 1;
+    if (per == 32) {
+        const bool is_long = j1 - j0 >= 4 * MEAN_SHORT;
+        long long acc[3];
+        int emin;
+        const bool ok = run_sums<1>(pix, L, j0, is_long ? j0 : j1, 0, acc, emin);
+        if (j1 > j0 && !is_long) {
             if (ok) {
-#pragma unroll
-                for (int u = 0; u < VU; ++u)
-#pragma unroll
-                    for (int k = 0; k < 3; ++k) acc[k] = fipt_exact::add_term(acc[k], v[u][k], emin);
+                const double n = (double)(j1 - j0);
+                grid[keys[j0]] = make_float4((float)(fipt_exact::scaled_double(acc[0], emin) / n),
+                                             (float)(fipt_exact::scaled_double(acc[1], emin) / n),
+                                             (float)(fipt_exact::scaled_double(acc[2], emin) / n), (float)n);
+            } else {
+                wide[atomicAdd(&n_wide, 1)] = make_uint2(j0, j1);
             }
         }
-        // the run's range and sums over its lanes
+        todo = __ballot_sync(FULL, is_long);
+    }
+    while (todo) {
+        if (per == 32) {                                   // four of the long ones
+            int of = -1;
 #pragma unroll
-        for (int o = 1; o < MEAN_LANES; o <<= 1) {
-            run.lo = min(run.lo, __shfl_xor_sync(FULL, run.lo, o));
-            run.hi = max(run.hi, __shfl_xor_sync(FULL, run.hi, o));
+            for (int g = 0; g < 32 / MEAN_LANES; ++g) {
+                if (lane / MEAN_LANES == g) of = __ffs(todo) - 1;
+                todo &= todo - 1;
+            }
+            r0 = __shfl_sync(FULL, j0, of & 31);
+            r1 = __shfl_sync(FULL, j1, of & 31);
+            if (of < 0) r1 = r0;
+        } else {
+            todo = 0;
         }
-        const unsigned lanes = ((1u << MEAN_LANES) - 1u) << (threadIdx.x & 31 & ~(MEAN_LANES - 1));
-        ok = (__ballot_sync(FULL, ok) & lanes) == lanes && !run.special() && run.exact_for(count);
-        const int least = run.emin();
-        const int sh = ok ? emin - least : 0;              // 0 to 29 where the lane has a nonzero value
-        double s = 0.0;                                    // lane k: channel k's sum
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            long long a = acc[k] == 0 ? 0 : (long long)((unsigned long long)acc[k] << min(sh, 63));
-#pragma unroll
-            for (int o = 1; o < MEAN_LANES; o <<= 1) a += __shfl_xor_sync(FULL, a, o);
-            if (c == k && ok) s = fipt_exact::scaled_double(a, least);
+        long long acc[3];
+        int emin;
+        const bool ok = run_sums<MEAN_LANES>(pix, L, r0, r1, c, acc, emin);
+        if (r1 > r0 && ok && c < 4) {                      // lanes 0 to 2 divide a channel each
+            const double s = fipt_exact::scaled_double(c == 0 ? acc[0] : c == 1 ? acc[1] : acc[2], emin);
+            reinterpret_cast<float*>(grid + keys[r0])[c] = c < 3 ? (float)(s / (double)(r1 - r0)) : (float)(r1 - r0);
         }
-        if (!ok && c < 3)
-            for (int64_t e = j0; e < j1; ++e) s += (double)L[3 * (int64_t)pix[e] + c];
-        const float m = c < 3 ? (float)(s / (double)(count > 0 ? count : 1)) : (float)count;
-        if (h < nh && c < 4) reinterpret_cast<float*>(grid + keys[j0])[c] = m;
+        if (r1 > r0 && !ok && c == 0) wide[atomicAdd(&n_wide, 1)] = make_uint2(r0, r1);
+    }
+    __syncthreads();
+    const int of = lane / 3, ch = lane - 3 * of;
+    for (int k = 10 * (threadIdx.x >> 5) + of; k < n_wide && of < 10; k += 10 * (MEAN_THREADS / 32)) {
+        const uint2 run = wide[k];
+        double s = 0.0;
+        uint32_t e = run.x;
+        for (; e + VU <= run.y; e += VU) {
+            float v[VU];
+#pragma unroll
+            for (int u = 0; u < VU; ++u) v[u] = L[3 * (int64_t)pix[e + u] + ch];
+#pragma unroll
+            for (int u = 0; u < VU; ++u) s += (double)v[u];
+        }
+        for (; e < run.y; ++e) s += (double)L[3 * (int64_t)pix[e] + ch];
+        float* g = reinterpret_cast<float*>(grid + keys[run.x]);
+        g[ch] = (float)(s / (double)(run.y - run.x));
+        if (ch == 0) g[3] = (float)(run.y - run.x);
     }
 }
 
@@ -309,9 +385,9 @@ extern "C" fipt_status fipt_voxel_cache_build(fipt_scene* s, const float* x, int
     FIPT_LAUNCH(k_vox_count, (unsigned)nt, HEAD_TILE, 0, st, sk, P, Y.tcount);
     FIPT_LAUNCH(k_vox_scan, 1, HEAD_TILE, 0, st, Y.tcount, nt, Y.heads, Y.nhead, P);
     FIPT_LAUNCH(k_vox_compact, (unsigned)nt, HEAD_TILE, 0, st, sk, P, Y.tcount, Y.heads);
-    // one run per thread at most (there are at most P runs)
+    // a thread per pixel: lanes enough for MEAN_LANES a run where runs have as many pixels, or one a run
     const unsigned mean_blocks = (unsigned)((P + MEAN_THREADS - 1) / MEAN_THREADS);
-    FIPT_LAUNCH(k_vox_means, mean_blocks, MEAN_THREADS, 0, st, sk, sv, Y.heads, Y.nhead, L,
+    FIPT_LAUNCH(k_vox_means, mean_blocks, MEAN_THREADS, 0, st, sk, sv, Y.heads, Y.nhead, P, L,
                 reinterpret_cast<float4*>(grid));
     FIPT_LAUNCHED("voxel cache build");
     return FIPT_OK;
