@@ -82,7 +82,9 @@ typedef struct fipt_query {
  *  K, sigma[K]: roughness levels (Eq. 8), each in (0, 1]; alpha = sigma^2.
  *  stats: NULL, or a device pointer to 4 unsigned 64-bit counters to which
  *    the bake ADDS: rays traced, BVH nodes visited, triangles tested, and
- *    (max, not added) the deepest traversal stack seen. */
+ *    (max, not added) the deepest traversal stack seen.  A stack holds 32
+ *    entries and is cut back to them every 8 visits, so a value of up to 40
+ *    can be seen; a ray that was cut back raises FIPT_DEV_STACK_OVERFLOW. */
 typedef struct fipt_bake_params {
     uint64_t seed;
     uint32_t request_id;
