@@ -84,7 +84,7 @@ struct fipt_scene {
     bool restructured = false;    // fipt_scene_optimize / relayout ran (range[] is the radix tree's only)
     BvhNode* nodes_alt = nullptr; // second node array (relayout target)
     int32_t* scratch = nullptr;   // [3 (T-1)] relayout scratch: subtree sizes, new indices, new parents
-    bool has_sizes = false;       // the scratch holds the tree's subtree sizes
+    bool has_sizes = false;       // the work enqueued so far leaves the tree's subtree sizes in the scratch
     const float* env = nullptr;   // caller-owned environment map
     int env_w = 0, env_h = 0;
     const float4* vox = nullptr;  // caller-owned voxel radiance cache

@@ -1262,6 +1262,8 @@ extern "C" fipt_status fipt_scene_optimize(fipt_scene* s, int32_t passes, fipt_s
     if (T < 3 || passes == 0) return FIPT_OK;
     FIPT_CUDA(cudaSetDevice(s->ctx->device));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    FIPT_CUDA(cudaStreamIsCapturing(st, &capture));
     for (int k = 0; k < passes; ++k) {
         FIPT_CUDA(cudaMemsetAsync(s->flags, 0, sizeof(int32_t) * (size_t)(T - 1), st));
         FIPT_LAUNCH(k_treelets, grid_for(T, TL_THREADS), TL_THREADS, 0, st, s->nodes, s->parent, s->leaf_parent, s->flags,
@@ -1269,7 +1271,7 @@ extern "C" fipt_status fipt_scene_optimize(fipt_scene* s, int32_t passes, fipt_s
     }
     FIPT_LAUNCHED("treelet restructuring");
     s->restructured = true;
-    s->has_sizes = true;
+    s->has_sizes = capture == cudaStreamCaptureStatusNone;     // a captured pass may run later, or never
     return FIPT_OK;
 }
 
