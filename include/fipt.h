@@ -620,6 +620,12 @@ fipt_status fipt_debug_divide(uint32_t n, const uint32_t* i, int64_t count, uint
  * the kernel's duration.  1 <= wait_polls <= 65536. */
 fipt_status fipt_debug_serve_wait_bound(int32_t wait_polls, int32_t* quit, int32_t* orphans,
                                         int32_t* warps, double* seconds);
+/* log2 of the lanes that share each of a bake's `pairs` (point, lobe) pairs on a
+ * GPU of `sms` SMs (the rule of fipt_bake, computed on the host; results do
+ * not depend on it).  -> *log_lanes in [0, 5].  Check entry point; no
+ * counterpart in the paper. */
+fipt_status fipt_debug_bake_split(int64_t pairs, int64_t T, int32_t spp_diffuse, int32_t spp_specular,
+                                  int32_t sms, int32_t* log_lanes);
 /* The order the server gives a bake's points (the order of
  * fipt_query_order, computed on the host by a threaded radix sort): q [n]
  * HOST, lo [3] / hi [3] HOST box -> order [n] HOST.  Check entry point; no

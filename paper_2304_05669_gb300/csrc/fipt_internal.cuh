@@ -189,9 +189,10 @@ struct ServeCounters {
     int pad;
 };
 
-// log2 of the lanes that share each of `pairs` (point, lobe) pairs of a bake in
-// a scene of T triangles, on the current device; at most one lane a sample.
-int bake_split(int64_t pairs, int64_t T, int least_spp);
+// log2 of the lanes that share each of `pairs` (point, lobe) pairs of a bake of
+// spp_d / spp_s samples in a scene of T triangles, on the current device; at most
+// one lane a sample.
+int bake_split(int64_t pairs, int64_t T, int spp_d, int spp_s);
 // Warp items of n points and L lobes at that split.
 __host__ __device__ inline int64_t bake_warps(int64_t n, int L, int log_g) {
     const int64_t per = 32 >> log_g;

@@ -582,8 +582,9 @@ void fipt_server::stage_chunks() {
         // with other requests to fill the chip, a small one gains nothing from spreading
         const int least = std::min(P.spp_diffuse, P.spp_specular);
         const int64_t T = scenes[q->r.target]->T;
-        const int log_g = std::min(bake_split(q->r.n * (1 + P.K), T, least),
-                                   std::max(bake_split(pairs_waiting, T, least), std::min(least, 2) - 1));
+        const int log_g = std::min(bake_split(q->r.n * (1 + P.K), T, P.spp_diffuse, P.spp_specular),
+                                   std::max(bake_split(pairs_waiting, T, P.spp_diffuse, P.spp_specular),
+                                            std::min(least, 2) - 1));
         int64_t got = 0;
         while (q->next < q->r.n && n_staged < kQueue) {
             const int64_t c = std::min<int64_t>(chunk_points, q->r.n - q->next);

@@ -5,6 +5,7 @@
 // tree, a ray per lane, the warp's lanes in step between inner nodes and
 // leaves, the stack in local memory.
 #include <algorithm>
+#include <climits>
 
 #include "fipt_internal.cuh"
 #include "render_math.cuh"
@@ -914,15 +915,27 @@ extern "C" fipt_status fipt_query_order(fipt_scene* s, const fipt_query* q, int6
 //   4,096 x 64 (0.09)                    0.84  0.48  0.33  0.30  0.30  0.36
 //   20,011 x 64 (0.45)                   1.14  0.91  0.82  0.79  0.86  1.20
 //   1,000,003 x 32 with a sky (16.1)     16.2  16.8  17.2  18.8  23.1  36.7
-int bake_split(int64_t pairs, int64_t T, int least_spp) {
+static int bake_split_on(int sms, int64_t pairs, int64_t T, int spp_d, int spp_s) {
+    const double fills = (double)pairs / (2048.0 * sms) * (T < 4096 ? 3.0 : 1.0);
+    int g = fills < 0.1 ? 5 : fills < 1.0 ? 4 : fills < 3.0 ? 3 : fills < 12.0 ? 2 : fills < 60.0 ? 1 : 0;
+    while ((1 << g) > std::min(spp_d, spp_s)) --g;                       // no lane without a sample
+    while (std::max(spp_d, spp_s) > INT_MAX - (1 << g) + 1) --g;         // a lane's next sample is an int
+    return g;
+}
+
+int bake_split(int64_t pairs, int64_t T, int spp_d, int spp_s) {
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
         return 0;
-    const double fills = (double)pairs / (2048.0 * sms) * (T < 4096 ? 3.0 : 1.0);
-    int g = fills < 0.1 ? 5 : fills < 1.0 ? 4 : fills < 3.0 ? 3 : fills < 12.0 ? 2 : fills < 60.0 ? 1 : 0;
-    while ((1 << g) > least_spp) --g;             // no lane without a sample
-    return g;
+    return bake_split_on(sms, pairs, T, spp_d, spp_s);
+}
+
+extern "C" fipt_status fipt_debug_bake_split(int64_t pairs, int64_t T, int32_t spp_diffuse, int32_t spp_specular,
+                                             int32_t sms, int32_t* log_lanes) {
+    FIPT_REQUIRE(log_lanes && pairs >= 1 && T >= 0 && spp_diffuse >= 1 && spp_specular >= 1 && sms >= 1, "bad arguments");
+    *log_lanes = bake_split_on(sms, pairs, T, spp_diffuse, spp_specular);
+    return FIPT_OK;
 }
 
 extern "C" fipt_status fipt_bake(fipt_scene* s, const fipt_query* q, int64_t N,
@@ -950,7 +963,7 @@ extern "C" fipt_status fipt_bake(fipt_scene* s, const fipt_query* q, int64_t N,
     A.K = prm->K;
     set_strata(A);
     for (int k = 0; k < FIPT_MAX_K; ++k) A.sigma[k] = k < prm->K ? prm->sigma[k] : 1.0f;
-    const int log_g = bake_split(N * (1 + prm->K), s->T, std::min(prm->spp_diffuse, prm->spp_specular));
+    const int log_g = bake_split(N * (1 + prm->K), s->T, prm->spp_diffuse, prm->spp_specular);
     const int64_t threads = 32 * bake_warps(N, 1 + prm->K, log_g);
     const unsigned nb = blocks(threads, BAKE_THREADS);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
