@@ -189,6 +189,10 @@ struct ServeCounters {
     int pad;
 };
 
+// Triangles under which a tree's walks are short beside what surrounds them
+// (measured at bake_split).
+constexpr int64_t BAKE_SMALL_TREE = 512;
+
 // log2 of the lanes that share each of `pairs` (point, lobe) pairs of a bake of
 // spp_d / spp_s samples in a scene of T triangles, on the current device; at most
 // one lane a sample.

@@ -915,8 +915,17 @@ extern "C" fipt_status fipt_query_order(fipt_scene* s, const fipt_query* q, int6
 //   4,096 x 64 (0.09)                    0.84  0.48  0.33  0.30  0.30  0.36
 //   20,011 x 64 (0.45)                   1.14  0.91  0.82  0.79  0.86  1.20
 //   1,000,003 x 32 with a sky (16.1)     16.2  16.8  17.2  18.8  23.1  36.7
+// Where a tree stops being small: a box with spheres, surface points in random
+// order, the rule's time over the best of the six at 0.09 / 0.45 / 1.6 / 5 / 20
+// fills, counted thrice and once:
+//   14 triangles     1.08  1.01  1.00  1.00  1.00      1.48  1.18  1.06  1.02  1.03
+//   334              1.00  1.00  1.00  1.04  1.02      1.14  1.04  1.00  1.00  1.00
+//   1,294            1.00  1.02  1.01  1.05  1.03      1.03  1.00  1.00  1.00  1.00
+//   2,574            1.00  1.04  1.03  1.06  1.05      1.02  1.00  1.00  1.00  1.01
+//   5,134            1.00  1.01  1.02  1.05  1.04      1.05  1.00  1.00  1.00  1.00
+//   20,494           1.09  1.07  1.06  1.09  1.10      1.00  1.00  1.01  1.02  1.04
 static int bake_split_on(int sms, int64_t pairs, int64_t T, int spp_d, int spp_s) {
-    const double fills = (double)pairs / (2048.0 * sms) * (T < 4096 ? 3.0 : 1.0);
+    const double fills = (double)pairs / (2048.0 * sms) * (T < BAKE_SMALL_TREE ? 3.0 : 1.0);
     int g = fills < 0.1 ? 5 : fills < 1.0 ? 4 : fills < 3.0 ? 3 : fills < 12.0 ? 2 : fills < 60.0 ? 1 : 0;
     while ((1 << g) > std::min(spp_d, spp_s)) --g;                       // no lane without a sample
     while (std::max(spp_d, spp_s) > INT_MAX - (1 << g) + 1) --g;         // a lane's next sample is an int
