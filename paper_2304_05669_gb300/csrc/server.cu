@@ -549,6 +549,26 @@ void fipt_server::untaken(int64_t* items, int64_t* rays) {
     *rays = r;
 }
 
+// log2 of the lanes a pair up to which a request's bake items are worth their
+// taking.  An item costs the loop two counters that all warps add to and a word of
+// host memory, some 25 M items a second in all, whatever it holds.  So splitting
+// goes on while the request has at most an item per resident warp (they would wait
+// otherwise), and beyond that while a lane keeps 4 samples, 16 in a small tree, whose
+// walks are short.  Requests of n points x spp samples x 7 lobes at once, ms with a
+// lane a pair / split without this limit / with it:
+//   Cornell box  10,000 x 16, 8 of them    1.72   3.19   1.63
+//                10,000 x 64, 20 of them   8.54  10.14   7.28
+//                50,000 x 16, one          1.46   1.47   1.37
+//   room         20,000 x 16, 8 of them    7.88   7.45   6.06
+//                10,000 x 64, 8 of them   17.05  10.70  10.75
+//                300 x 16, one             1.38   0.43   0.43
+static int item_split(int64_t pairs, int64_t T, int least_spp, int64_t resident_warps) {
+    const int keep = T < BAKE_SMALL_TREE ? 16 : 4;
+    int g = 0;
+    while (g < 5 && (pairs * (2 << g) <= 32 * resident_warps || (int64_t)keep * (2 << g) <= least_spp)) ++g;
+    return g;
+}
+
 // Stages chunk descriptors while fewer than lookahead_items warp items (two
 // per resident warp of the loop) and fewer than lookahead_rays rays are
 // published and not yet taken: the oldest admitted bake first, up to a
@@ -579,12 +599,14 @@ void fipt_server::stage_chunks() {
         const fipt_bake_params& P = q->r.params;
         const int64_t rpp = rays_per_point(P);
         // the request's own split, but no finer than two lanes a pair where the work waiting would not want it:
-        // with other requests to fill the chip, a small one gains nothing from spreading
+        // with other requests to fill the chip, a small one gains nothing from spreading; and no finer than its items
+        // are worth their taking
         const int least = std::min(P.spp_diffuse, P.spp_specular);
         const int64_t T = scenes[q->r.target]->T;
-        const int log_g = std::min(bake_split(q->r.n * (1 + P.K), T, P.spp_diffuse, P.spp_specular),
-                                   std::max(bake_split(pairs_waiting, T, P.spp_diffuse, P.spp_specular),
-                                            std::min(least, 2) - 1));
+        const int log_g = std::min({bake_split(q->r.n * (1 + P.K), T, P.spp_diffuse, P.spp_specular),
+                                    std::max(bake_split(pairs_waiting, T, P.spp_diffuse, P.spp_specular),
+                                             std::min(least, 2) - 1),
+                                    item_split(q->r.n * (1 + P.K), T, least, lookahead_items / 2)});
         int64_t got = 0;
         while (q->next < q->r.n && n_staged < kQueue) {
             const int64_t c = std::min<int64_t>(chunk_points, q->r.n - q->next);
