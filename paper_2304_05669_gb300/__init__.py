@@ -28,11 +28,16 @@ def _ptr(t):
     return t.data_ptr() if t is not None else None
 
 
+# the current stream's handle without the Stream object around it (10 us on the GB300's host cores); not a public name
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream=None):
     if stream is not None:
         return stream.cuda_stream
-    # the current stream's handle without the Stream object around it (10 us on the GB300's host cores)
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    if _raw_stream is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(torch.cuda.current_device())
 
 
 def _dev(t, dtype, name):
