@@ -690,7 +690,7 @@ __device__ __forceinline__ void best_split(const float* cl, const float* cr, int
 }
 
 // Restructures the treelet rooted at p; all 32 lanes of the warp call it
-// with the same p.  Lane i holds treelet leaf i and internal node i.  The
+// with the same p, which has an internal child.  Lane i holds treelet leaf i and internal node i.  The
 // kernel is bound by the instructions it issues, so every part is spread over
 // the lanes: the area of the 127 subsets (a lane unites the leaves of its
 // index's five bits once and adds the four combinations of the last two), the
@@ -736,8 +736,9 @@ __device__ void restructure_warp(BvhNode* nodes, int32_t* parent, int32_t* leaf_
     float cur = __shfl_sync(FULL, half_area(box_union(box, other)), 0);   // the current internal areas
     int m = 2;
     while (m < TREELET) {
-        // the internal leaf of largest area, the first one on a tie
-        const unsigned key = ref >= 0 && area > -1.0f ? (__float_as_uint(area) & 0x7fffffffu) + 1u : 0u;
+        // the internal leaf of largest area, the first one on a tie; before all others one whose area is NaN (infinity
+        // times zero), so that p, which has an internal child, comes to three leaves whatever the boxes
+        const unsigned key = ref >= 0 ? (__float_as_uint(area) & 0x7fffffffu) + 1u : 0u;
         const unsigned top = __reduce_max_sync(FULL, key);
         if (top == 0) break;
         const int best = __ffs(__ballot_sync(FULL, key == top)) - 1;
@@ -747,15 +748,14 @@ __device__ void restructure_warp(BvhNode* nodes, int32_t* parent, int32_t* leaf_
         if (lane == best || lane == m) take_child(n, lane == m);
         ++m;
     }
+    if (m < 3) return;                                     // p has no internal child: not called so
     if (size) {
         const int below = lane < m && ref >= 0 ? __ldcg(size + ref) : 0;
         if (lane < m) tb.size[lane] = below;
         const int all = __reduce_add_sync(FULL, below) + m - 1;
         if (lane == 0) __stcg(size + p, all);              // whatever the topology
     }
-    // nothing changed, or two leaves: one topology (internal leaves whose box has no area to compare, infinity times
-    // zero, stay closed)
-    if (m < 3 || !__any_sync(FULL, fresh)) {
+    if (!__any_sync(FULL, fresh)) {
         __syncwarp();
         return;
     }
