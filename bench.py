@@ -653,7 +653,7 @@ def run_refine(args, F, dev, mesh, sc, q_all, with_cpu):
                         "unit": "GB/s", "frac": round(alg / t / 1e9 / peak, 4), "peak_kind": peak_kind,
                         "kernel": "whole call: k_rf_gen, k_rf_trace, k_rf_shade, k_rf_reduce",
                         "note": "algorithmic node + triangle + gather + path-state bytes / call time; the "
-                                "traversal (75 % of the call) is served by L1/L2 and bound by issue"}}
+                                "traversal (75 % of the call) is served by L1/L2 and bound by L1's data pipe, then by issue"}}
     if with_cpu:
         import oracle as O
         cams = pinhole_views_for(mesh)
@@ -856,7 +856,7 @@ def bake_roofline(prof, rays_per_step, n_rays_traced, alg_bytes, bake_s, sm_mhz,
             "unit": "Gwarp-inst/s", "frac": round(ach_issue / peak_issue, 4),
             "traffic": int(round(traffic)), "kernel": "k_bake",
             "peak_kind": "derived: %d SMs x 4 schedulers x %.0f MHz sampled SM clock" % (n_sm, sm_mhz),
-            "what": "warp-instruction issue (the walk is bound by issue and divergence, not by HBM)",
+            "what": "warp-instruction issue (after L1's data pipe the walk's bound; not HBM)",
             "warp_inst_per_ray": round(float(prof["warp_inst_per_ray"]), 2),
             "lanes_per_warp_inst": lanes,
             "lane_frac": round(ach_issue / peak_issue * lanes / 32.0, 4),

@@ -253,10 +253,10 @@ fipt_status fipt_bake(fipt_scene* scene, const fipt_query* q, int64_t N,
  * order [N] DEVICE int32 receives the indices of the points sorted by the
  * 30-bit Morton code of their positions in the scene's bounding box
  * (stable: equal codes keep index order).  A warp bakes 32 consecutive
- * slots, and with this order its points lie close together, so their rays
- * start near each other and walk the tree alike (about 7 % faster on the
- * building floor than compacted pixel order; random order halves the
- * rate).  Workspace: fipt_query_order_workspace_size, 256-byte aligned. */
+ * slots (fewer where lanes share a point), and with this order its points
+ * lie close together, so their rays start near each other and walk the tree
+ * alike (about 7 % faster on the building floor than compacted pixel order;
+ * random order halves the rate).  Workspace: fipt_query_order_workspace_size, 256-byte aligned. */
 fipt_status fipt_query_order_workspace_size(int64_t N, size_t* bytes);
 fipt_status fipt_query_order(fipt_scene* scene, const fipt_query* q, int64_t N, int32_t* order,
                              void* workspace, size_t ws_bytes, fipt_stream stream);

@@ -142,7 +142,7 @@ def unpack_queries(q):
 OPTIMIZE_PASSES = 2      # treelet-restructuring passes a Scene gets by default ...
 OPTIMIZE_MIN_TRIS = 4096  # ... from this many triangles (smaller trees stay cache-resident)
 OPTIMIZE_PASSES_LARGE = 3  # ... and from OPTIMIZE_LARGE_TRIS on: on a 2M-triangle floor
-OPTIMIZE_LARGE_TRIS = 1 << 20  # a third pass (7 ms) saves 1.5 % of the node visits per ray
+OPTIMIZE_LARGE_TRIS = 1 << 20  # a third pass (1.4 ms) saves 1.5 % of the node visits per ray
 RELAYOUT = True           # depth-first node renumbering after the passes
 
 

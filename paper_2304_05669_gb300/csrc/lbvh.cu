@@ -50,7 +50,7 @@ __device__ __forceinline__ uint4 load4(const uint32_t* a, int64_t i, int64_t m) 
 }
 
 // The block's exclusive scan of its threads' t, plus base; total receives the
-// sum.  wsum: 33 words.
+// sum.  wsum: a word per warp.
 __device__ __forceinline__ uint32_t scan_threads(uint32_t t, uint32_t base, uint32_t* wsum, uint32_t& total) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t incl = t;

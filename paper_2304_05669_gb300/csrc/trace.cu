@@ -212,8 +212,6 @@ k_compact(const fipt_query* __restrict__ in, const int32_t* __restrict__ valid, 
 #endif
 constexpr int BAKE_THREADS = FIPT_BAKE_THREADS;
 
-
-
 // Bakes one (point, lobe) pair per lane: lobe 0 is the diffuse term, lobe
 // k+1 roughness level k.  Each lane walks its pair's samples in order and
 // sums their contributions in that order (so the result does not depend on
@@ -567,6 +565,30 @@ __device__ __noinline__ int serve_take_bake(ServeShared* sh, ServeCounters* ctr,
     }
 }
 
+// A value all lanes of the warp hold, as one the compiler knows they do (the
+// reduction's result is a uniform register).  The serving loop's scene comes
+// from its chunk's descriptor, not from kernel parameters: the walk would load
+// its pointers and sizes again on every visit, through an L1 that is its bound
+// (500 mixed requests in the loop: 4,855 -> 5,123 Mrays/s).
+__device__ __forceinline__ int uniform(int v) { return (int)__reduce_or_sync(0xffffffffu, (unsigned)v); }
+template <class P>
+__device__ __forceinline__ const P* uniform(const P* p) {
+    const unsigned long long v = reinterpret_cast<unsigned long long>(p);
+    return reinterpret_cast<const P*>((unsigned long long)(unsigned)uniform((int)(v >> 32)) << 32 |
+                                      (unsigned)uniform((int)v));
+}
+__device__ __forceinline__ SceneView uniform_scene(const SceneView& sc) {
+    SceneView u = sc;
+    u.nodes = uniform(sc.nodes);
+    u.tris = uniform(sc.tris);
+    u.shade = uniform(sc.shade);
+    u.cst = uniform(sc.cst);
+    u.T = (int64_t)uniform((int)sc.T);
+    u.n_inner = uniform(sc.n_inner);
+    u.max_steps = uniform(sc.max_steps);
+    return u;
+}
+
 // The server's bake loop: resident warps take bake items (32 / G points of one
 // chunk, one lobe, G = 2^log_g lanes a pair) in publication order from a device counter with one
 // atomicAdd each (no compare-and-swap retries, so thousands of warps do not
@@ -593,30 +615,6 @@ __device__ __noinline__ int serve_take_bake(ServeShared* sh, ServeCounters* ctr,
 // requests have a loop of their own (k_serve_render) beside this one: code
 // for them in this kernel cost the bake walk 7 % through its register
 // allocation.
-// A value all lanes of the warp hold, as one the compiler knows they do (the
-// reduction's result is a uniform register).  The serving loop's scene comes
-// from its chunk's descriptor, not from kernel parameters: the walk would load
-// its pointers and sizes again on every visit, through an L1 that is its bound
-// (500 mixed requests in the loop: 4,855 -> 5,123 Mrays/s).
-__device__ __forceinline__ int uniform(int v) { return (int)__reduce_or_sync(0xffffffffu, (unsigned)v); }
-template <class P>
-__device__ __forceinline__ const P* uniform(const P* p) {
-    const unsigned long long v = reinterpret_cast<unsigned long long>(p);
-    return reinterpret_cast<const P*>((unsigned long long)(unsigned)uniform((int)(v >> 32)) << 32 |
-                                      (unsigned)uniform((int)v));
-}
-__device__ __forceinline__ SceneView uniform_scene(const SceneView& sc) {
-    SceneView u = sc;
-    u.nodes = uniform(sc.nodes);
-    u.tris = uniform(sc.tris);
-    u.shade = uniform(sc.shade);
-    u.cst = uniform(sc.cst);
-    u.T = (int64_t)uniform((int)sc.T);
-    u.n_inner = uniform(sc.n_inner);
-    u.max_steps = uniform(sc.max_steps);
-    return u;
-}
-
 template <int FLAGS>
 __global__ void __launch_bounds__(BAKE_THREADS, FIPT_BAKE_MINB)
 k_serve_bake(const BakeChunk* __restrict__ chunks, ServeShared* sh, ServeCounters* ctr,
