@@ -154,7 +154,9 @@ k_vox_compact(const uint32_t* __restrict__ keys, int64_t P, const uint32_t* __re
 
 constexpr int MEAN_THREADS = 128;
 constexpr int MEAN_LANES = 8;    // lanes per run where the runs are long
-constexpr int MEAN_SHORT = 8;    // pixels per run, on average, from which they are
+constexpr int MEAN_UNIT = MEAN_THREADS / MEAN_LANES;     // runs of a block there
+constexpr int MEAN_SUBS = MEAN_THREADS / MEAN_UNIT;      // and such blocks per run of each thread
+constexpr int MEAN_SHORT = 4;    // pixels per run, over MEAN_THREADS neighbouring runs, up to which they are short
 constexpr int VU = 4;            // pixels a lane takes at a time
 
 // The sums of one run per LANES lanes (lane c of them, run [j0, j1) of count
@@ -239,89 +241,104 @@ __device__ __forceinline__ bool run_sums(const uint32_t* __restrict__ pix, const
 // Means of the runs.  Long runs take MEAN_LANES lanes each, as the kernel is
 // bound by its longest ones (4,194,304 pixels of the room in 256^3 cells, 14 a
 // run: 210 us with a lane per run, 17 % of the warps active -> 62 us), then by
-// the gathers.  Where a run has under MEAN_SHORT pixels on average most of those
-// lanes would idle: a warp takes 32 runs, a lane each, and then the long ones among
-// them as before (4,194,304 points in 256^3 cells, 1.1 a run: the whole call 906 us
-// with MEAN_LANES for all, 548 with a lane for all, 494).
+// the gathers.  Where MEAN_THREADS neighbouring runs are short most of those
+// lanes would idle, and one of their MEAN_SUBS blocks takes them all, a lane each,
+// and then the long ones among them as before (4,000,000 points in 256^3 cells,
+// 1.1 a run: the whole call 903 us with MEAN_LANES for all, 546 with a lane for
+// all, 508).  The choice is made by neighbourhood, as dense cells lie side by side
+// and a block that took 128 long runs would work them off one after the other
+// (813,120 pixels of a floor in 256^3 cells, 4.2 a run and up to 1,447: 206 us with
+// MEAN_LANES for all, 258 with a lane for all under 32 pixels, 201).  MEAN_SHORT 3 /
+// 4 / 6 / 8 over 118 calls of 1 to 70 pixels a run: on average 1.03 / 1.05 / 1.05 / 1.05
+// times as fast as the faster of one kind for all, at worst 0.98 / 0.99 / 0.97 / 0.95.
 //
 // Runs outside the exact range are listed by their block, which then adds up
 // ten of them a warp, every lane a channel of one, in FP64 in pixel order
 // (4,194,304 points in 64^3 cells, all outside it: 403 us with a lane a run, 480
-// with three lanes of MEAN_LANES, 400).  There is a thread per pixel, so a warp
-// for every `per` runs.
+// with three lanes of MEAN_LANES, 400).
 __global__ void __launch_bounds__(MEAN_THREADS)
 k_vox_means(const uint32_t* __restrict__ keys, const uint32_t* __restrict__ pix, const uint32_t* __restrict__ heads,
-            const uint32_t* __restrict__ nhead, int64_t P, const float* __restrict__ L, float4* __restrict__ grid) {
+            const uint32_t* __restrict__ nhead, const float* __restrict__ L, float4* __restrict__ grid) {
     constexpr unsigned FULL = 0xffffffffu;
     __shared__ uint2 wide[MEAN_THREADS];                   // [j0, j1) of the block's runs outside the exact range
     __shared__ int n_wide;
-    const int nh = (int)*nhead;
-    const int per = P >= MEAN_SHORT * (int64_t)nh ? 32 / MEAN_LANES : 32;      // runs a warp takes
-    if ((int64_t)blockIdx.x * (MEAN_THREADS / 32) * per >= nh) return;         // whole block
+    const int nh = (int)*nhead, units = (nh + MEAN_UNIT - 1) / MEAN_UNIT;
+    const int lane = threadIdx.x & 31, c = lane % MEAN_LANES;
     if (threadIdx.x == 0) n_wide = 0;
     __syncthreads();
-    const int lane = threadIdx.x & 31, c = lane % MEAN_LANES;
-    const int h = (int)(blockIdx.x * (MEAN_THREADS / 32) + (threadIdx.x >> 5)) * per + (per == 32 ? lane : lane / MEAN_LANES);
-    const uint32_t j0 = h < nh ? heads[h] : 0, j1 = h < nh ? heads[h + 1] : 0;     // empty past nh
-    uint32_t r0 = j0, r1 = j1;
-    unsigned todo = 1;
-    if (per == 32) {
-        const bool is_long = j1 - j0 >= 4 * MEAN_SHORT;
-        long long acc[3];
-        int emin;
-        const bool ok = run_sums<1>(pix, L, j0, is_long ? j0 : j1, 0, acc, emin);
-        if (j1 > j0 && !is_long) {
-            if (ok) {
-                const double n = (double)(j1 - j0);
-                grid[keys[j0]] = make_float4((float)(fipt_exact::scaled_double(acc[0], emin) / n),
-                                             (float)(fipt_exact::scaled_double(acc[1], emin) / n),
-                                             (float)(fipt_exact::scaled_double(acc[2], emin) / n), (float)n);
-            } else {
-                wide[atomicAdd(&n_wide, 1)] = make_uint2(j0, j1);
-            }
+    for (int u = blockIdx.x; u < units; u += gridDim.x) {
+        // the block's neighbourhood, and which of its blocks works where it is short (another one in each, so that a
+        // block that goes round several times works in one of MEAN_SUBS)
+        const int near = u / MEAN_SUBS, n0 = near * MEAN_THREADS, n1 = min(nh, n0 + MEAN_THREADS);
+        int h = u * MEAN_UNIT + (int)threadIdx.x / MEAN_LANES;
+        uint32_t j0 = h < n1 ? heads[h] : 0, j1 = h < n1 ? heads[h + 1] : 0;     // empty past n1
+        const bool lanes = heads[n1] - heads[n0] <= (uint32_t)(MEAN_SHORT * (n1 - n0));
+        if (lanes) {
+            if (u % MEAN_SUBS != near % min(MEAN_SUBS, units - near * MEAN_SUBS)) continue;      // whole block
+            h = n0 + (int)threadIdx.x;
+            j0 = h < n1 ? heads[h] : 0;
+            j1 = h < n1 ? heads[h + 1] : 0;
         }
-        todo = __ballot_sync(FULL, is_long);
-    }
-    while (todo) {
-        if (per == 32) {                                   // four of the long ones
-            int of = -1;
-#pragma unroll
-            for (int g = 0; g < 32 / MEAN_LANES; ++g) {
-                if (lane / MEAN_LANES == g) of = __ffs(todo) - 1;
-                todo &= todo - 1;
+        const auto group = [&](uint32_t r0, uint32_t r1) {
+            long long acc[3];
+            int emin;
+            const bool ok = run_sums<MEAN_LANES>(pix, L, r0, r1, c, acc, emin);
+            if (r1 > r0 && ok && c < 4) {                  // lanes 0 to 2 divide a channel each
+                const double s = fipt_exact::scaled_double(c == 0 ? acc[0] : c == 1 ? acc[1] : acc[2], emin);
+                reinterpret_cast<float*>(grid + keys[r0])[c] = c < 3 ? (float)(s / (double)(r1 - r0)) : (float)(r1 - r0);
             }
-            r0 = __shfl_sync(FULL, j0, of & 31);
-            r1 = __shfl_sync(FULL, j1, of & 31);
-            if (of < 0) r1 = r0;
+            if (r1 > r0 && !ok && c == 0) wide[atomicAdd(&n_wide, 1)] = make_uint2(r0, r1);
+        };
+        if (!lanes) {
+            group(j0, j1);
         } else {
-            todo = 0;
-        }
-        long long acc[3];
-        int emin;
-        const bool ok = run_sums<MEAN_LANES>(pix, L, r0, r1, c, acc, emin);
-        if (r1 > r0 && ok && c < 4) {                      // lanes 0 to 2 divide a channel each
-            const double s = fipt_exact::scaled_double(c == 0 ? acc[0] : c == 1 ? acc[1] : acc[2], emin);
-            reinterpret_cast<float*>(grid + keys[r0])[c] = c < 3 ? (float)(s / (double)(r1 - r0)) : (float)(r1 - r0);
-        }
-        if (r1 > r0 && !ok && c == 0) wide[atomicAdd(&n_wide, 1)] = make_uint2(r0, r1);
-    }
-    __syncthreads();
-    const int of = lane / 3, ch = lane - 3 * of;
-    for (int k = 10 * (threadIdx.x >> 5) + of; k < n_wide && of < 10; k += 10 * (MEAN_THREADS / 32)) {
-        const uint2 run = wide[k];
-        double s = 0.0;
-        uint32_t e = run.x;
-        for (; e + VU <= run.y; e += VU) {
-            float v[VU];
+            const bool is_long = j1 - j0 >= 32;
+            long long acc[3];
+            int emin;
+            const bool ok = run_sums<1>(pix, L, j0, is_long ? j0 : j1, 0, acc, emin);
+            if (j1 > j0 && !is_long) {
+                if (ok) {
+                    const double n = (double)(j1 - j0);
+                    grid[keys[j0]] = make_float4((float)(fipt_exact::scaled_double(acc[0], emin) / n),
+                                                 (float)(fipt_exact::scaled_double(acc[1], emin) / n),
+                                                 (float)(fipt_exact::scaled_double(acc[2], emin) / n), (float)n);
+                } else {
+                    wide[atomicAdd(&n_wide, 1)] = make_uint2(j0, j1);
+                }
+            }
+            for (unsigned todo = __ballot_sync(FULL, is_long); todo;) {      // four of the long ones
+                int of = -1;
 #pragma unroll
-            for (int u = 0; u < VU; ++u) v[u] = L[3 * (int64_t)pix[e + u] + ch];
-#pragma unroll
-            for (int u = 0; u < VU; ++u) s += (double)v[u];
+                for (int g = 0; g < 32 / MEAN_LANES; ++g) {
+                    if (lane / MEAN_LANES == g) of = __ffs(todo) - 1;
+                    todo &= todo - 1;
+                }
+                const uint32_t r0 = __shfl_sync(FULL, j0, of & 31), r1 = __shfl_sync(FULL, j1, of & 31);
+                group(r0, of < 0 ? r0 : r1);
+            }
         }
-        for (; e < run.y; ++e) s += (double)L[3 * (int64_t)pix[e] + ch];
-        float* g = reinterpret_cast<float*>(grid + keys[run.x]);
-        g[ch] = (float)(s / (double)(run.y - run.x));
-        if (ch == 0) g[3] = (float)(run.y - run.x);
+        __syncthreads();
+        const int listed = n_wide, of = lane / 3, ch = lane - 3 * of;
+        for (int k = 10 * (threadIdx.x >> 5) + of; k < listed && of < 10; k += 10 * (MEAN_THREADS / 32)) {
+            const uint2 run = wide[k];
+            double s = 0.0;
+            uint32_t e = run.x;
+            for (; e + VU <= run.y; e += VU) {
+                float v[VU];
+#pragma unroll
+                for (int q = 0; q < VU; ++q) v[q] = L[3 * (int64_t)pix[e + q] + ch];
+#pragma unroll
+                for (int q = 0; q < VU; ++q) s += (double)v[q];
+            }
+            for (; e < run.y; ++e) s += (double)L[3 * (int64_t)pix[e] + ch];
+            float* g = reinterpret_cast<float*>(grid + keys[run.x]);
+            g[ch] = (float)(s / (double)(run.y - run.x));
+            if (ch == 0) g[3] = (float)(run.y - run.x);
+        }
+        if (u + (int)gridDim.x >= units) break;
+        __syncthreads();                                   // the list is read
+        if (threadIdx.x == 0) n_wide = 0;
+        __syncthreads();
     }
 }
 
@@ -385,9 +402,10 @@ extern "C" fipt_status fipt_voxel_cache_build(fipt_scene* s, const float* x, int
     FIPT_LAUNCH(k_vox_count, (unsigned)nt, HEAD_TILE, 0, st, sk, P, Y.tcount);
     FIPT_LAUNCH(k_vox_scan, 1, HEAD_TILE, 0, st, Y.tcount, nt, Y.heads, Y.nhead, P);
     FIPT_LAUNCH(k_vox_compact, (unsigned)nt, HEAD_TILE, 0, st, sk, P, Y.tcount, Y.heads);
-    // a thread per pixel: lanes enough for MEAN_LANES a run where runs have as many pixels, or one a run
-    const unsigned mean_blocks = (unsigned)((P + MEAN_THREADS - 1) / MEAN_THREADS);
-    FIPT_LAUNCH(k_vox_means, mean_blocks, MEAN_THREADS, 0, st, sk, sv, Y.heads, Y.nhead, P, L,
+    // a thread per pixel: a unit a block where runs have MEAN_LANES pixels, up to MEAN_SUBS where they have one; an odd
+    // multiple of MEAN_SUBS blocks, so that a block's units lie in neighbourhoods of all residues
+    const int64_t eighth = (P + MEAN_THREADS * MEAN_SUBS - 1) / (MEAN_THREADS * MEAN_SUBS) | 1;
+    FIPT_LAUNCH(k_vox_means, (unsigned)(MEAN_SUBS * eighth), MEAN_THREADS, 0, st, sk, sv, Y.heads, Y.nhead, L,
                 reinterpret_cast<float4*>(grid));
     FIPT_LAUNCHED("voxel cache build");
     return FIPT_OK;

@@ -1,6 +1,7 @@
-"""Voxel means where the runs are short on average: a lane a run, four long
-ones among them at a time, and runs outside the exact integer range held back
-until ten fill a warp; bit-equal to the oracle's grid."""
+"""Voxel means where neighbouring runs are short: a lane a run, four long ones
+among them at a time, dense neighbourhoods of 128 runs beside such ones (and a
+last one that is not full), and runs outside the exact integer range listed by
+their block; bit-equal to the oracle's grid."""
 import numpy as np
 import pytest
 import torch
@@ -12,15 +13,17 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("kind", ["narrow", "wide", "some wide", "signs"])
-@pytest.mark.parametrize("runs,long_runs", [(1, 0), (31, 0), (33, 1), (60, 5), (700, 4), (700, 17)])
-def test_short_runs(kind, runs, long_runs):
+@pytest.mark.parametrize("runs,long_runs,dense", [(1, 0, 0), (31, 0, 0), (129, 1, 0), (140, 2, 128), (700, 4, 0), (700, 7, 256),
+                                                  (1000, 9, 900)])
+def test_short_runs(kind, runs, long_runs, dense):
     import paper_2304_05669_gb300 as F
     rng = np.random.default_rng(runs + long_runs)
-    lengths = rng.integers(1, 5, runs)
-    lengths[rng.permutation(runs)[:long_runs]] = rng.choice([31, 32, 33, 65], long_runs)
-    assert lengths.sum() < 8 * runs                       # under the limit of the other path
     R = 32
-    cell = rng.permutation(np.repeat(rng.permutation(R * R)[:runs], lengths))
+    lengths = rng.integers(1, 4, runs)
+    lengths[rng.permutation(runs)[:long_runs]] = rng.choice([31, 32, 33, 65], long_runs)
+    lengths[:dense] += rng.integers(0, 40, dense)         # runs follow one another in the order of their cells
+    cells = np.sort(rng.permutation(R * R)[:runs])
+    cell = rng.permutation(np.repeat(cells, lengths))
     x = np.stack([(cell % R + 0.5) / R, (cell // R + 0.5) / R, np.full(len(cell), 0.5 / R)], 1).astype(np.float32)
     L = rng.uniform(0.25, 2.0, (len(cell), 3)).astype(np.float32)
     if kind == "wide":
