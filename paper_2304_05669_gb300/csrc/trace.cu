@@ -517,11 +517,16 @@ __device__ __forceinline__ void render_item(const RenderChunk& RC, int64_t il, i
 __device__ __forceinline__ double render_loss(const RenderChunk& RC, int lane) {
     using namespace fipt_render;
     const int64_t nb = (RC.n + RENDER_BLOCK - 1) / RENDER_BLOCK;
+    constexpr int SIDE = 8;                                // warps stood in for side by side: loads in flight
     double t = 0.0;
-    for (int j = 0; j < RENDER_SUM_THREADS / 32; ++j) {
-        double acc = 0.0;
-        for (int64_t i = j * 32 + lane; i < nb; i += RENDER_SUM_THREADS) acc += __ldcg(RC.partial + i);
-        t += warp_sum_down(acc);
+    for (int j = 0; j < RENDER_SUM_THREADS / 32; j += SIDE) {
+        double acc[SIDE] = {};
+        for (int64_t i = j * 32 + lane; i - lane < nb; i += RENDER_SUM_THREADS) {
+#pragma unroll
+            for (int k = 0; k < SIDE; ++k) acc[k] += i + 32 * k < nb ? __ldcg(RC.partial + i + 32 * k) : 0.0;
+        }
+#pragma unroll
+        for (int k = 0; k < SIDE; ++k) t += warp_sum_down(acc[k]);
     }
     return t;
 }
